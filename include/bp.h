@@ -380,7 +380,7 @@ int bp_assign_particles_part(bp_ctx* ctx, int64_t n, const float* x, const float
  *   select: BP_SELECT_ALL / HALO / FIELD
  *   ymap, bmap, ylo, blo: [ny][nx] FP32, accumulated (geom->n_maps must be 1).
  * Kernel support outside the map is dropped.  h = 0 deposits to the nearest grid
- * point.  Deterministic: particles are summed per tile in index order with
+ * point.  Deterministic: particles are summed per tile in a fixed order with
  * compensated FP32 sums.  Synchronises once to size the pair list. */
 int bp_paste_particles(bp_ctx* ctx, int64_t n, const float* assigned, const bp_map_geom* geom,
                        int select, float* ymap, float* bmap, float* ylo, float* blo);

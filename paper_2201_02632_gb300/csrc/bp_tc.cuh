@@ -2,7 +2,8 @@
 // tensor memory (TMEM) and shared-memory mbarriers, as used by the tensor-core deposit and
 // the surrogate's inference.
 //
-// Operand layout: K-major with the 128-byte swizzle.  A row holds 64 FP16 or BF16 values
+// Operand layouts, both with the 128-byte swizzle: MN-major (the deposit; desc_mn128) and
+// K-major (the inference; desc_sw128).  K-major:  A row holds 64 FP16 or BF16 values
 // (128 bytes); 8 rows form a 1024-byte atom; the 16-byte chunk q of row r sits at chunk
 // position q ^ (r % 8).  Atoms are stacked along M (or N) 1024 bytes apart.  One MMA
 // step covers K = 16 (32 bytes); step s starts 32 s bytes into the row.
@@ -13,15 +14,6 @@ namespace bptc {
 
 __device__ __forceinline__ uint32_t smem_u32(const void* p) {
   return (uint32_t)__cvta_generic_to_shared(p);
-}
-
-// byte offset of element (row r, k) in a K-major 128B-swizzled block, 0 <= k < 32
-__device__ __forceinline__ int sw128_off(int r, int k) {
-  return (r >> 3) * 1024 + (r & 7) * 128 + ((((k >> 2) ^ (r & 7))) << 4) + (k & 3) * 4;
-}
-// byte offset of the 16-byte chunk holding k = 4 kq .. 4 kq + 3 of row r
-__device__ __forceinline__ int sw128_quad(int r, int kq) {
-  return (r >> 3) * 1024 + (r & 7) * 128 + ((kq ^ (r & 7)) << 4);
 }
 
 // Shared-memory matrix descriptor: start address, leading offset 16 B (unused by the
@@ -49,6 +41,56 @@ __host__ __device__ constexpr uint32_t idesc_f16(int M, int N) {
   return (1u << 4) | ((uint32_t)(N >> 3) << 17) | ((uint32_t)(M >> 4) << 24);
 }
 
+// Instruction descriptor bits: A (B) is MN-major in shared memory instead of K-major.
+constexpr uint32_t IDESC_A_MN = 1u << 15, IDESC_B_MN = 1u << 16;
+
+// Matrix descriptor of an MN-major operand with the 128-byte swizzle: a 128-byte row holds 64
+// consecutive M (or N) elements of one k, 8 rows form a 1024-byte atom (16-byte chunk c of row
+// k at chunk c ^ (k % 8)); atoms follow 1024 bytes apart along K (stride offset) and mn_stride
+// bytes apart along M or N (leading offset).
+__device__ __forceinline__ uint64_t desc_mn128(uint32_t saddr, uint32_t mn_stride) {
+  uint64_t d = (uint64_t)((saddr >> 4) & 0x3FFF);
+  d |= (uint64_t)(mn_stride >> 4) << 16;
+  d |= (uint64_t)(1024 >> 4) << 32;
+  d |= (uint64_t)1 << 46;
+  d |= (uint64_t)2 << 61;
+  return d;
+}
+
+// ------------------------------------------------------------------ packed FP32 pairs
+// Two FP32 values per instruction, each operation rounded to nearest as its scalar form.
+__device__ __forceinline__ uint64_t f2_bits(float2 v) {
+  uint64_t r;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(v.x), "f"(v.y));
+  return r;
+}
+__device__ __forceinline__ float2 f2_vals(uint64_t b) {
+  float2 v;
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(v.x), "=f"(v.y) : "l"(b));
+  return v;
+}
+__device__ __forceinline__ float2 add2(float2 a, float2 b) {
+  uint64_t r;
+  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(f2_bits(a)), "l"(f2_bits(b)));
+  return f2_vals(r);
+}
+__device__ __forceinline__ float2 mul2(float2 a, float2 b) {
+  uint64_t r;
+  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(f2_bits(a)), "l"(f2_bits(b)));
+  return f2_vals(r);
+}
+__device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c) {
+  uint64_t r;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;"
+      : "=l"(r)
+      : "l"(f2_bits(a)), "l"(f2_bits(b)), "l"(f2_bits(c)));
+  return f2_vals(r);
+}
+// a - b, exactly rounded (b times -1 is exact)
+__device__ __forceinline__ float2 sub2(float2 a, float2 b) {
+  return fma2(b, make_float2(-1.f, -1.f), a);
+}
+
 // ------------------------------------------------------------------ mbarrier
 __device__ __forceinline__ void mbar_init(uint64_t* bar, uint32_t count) {
   asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(bar)), "r"(count));
@@ -62,6 +104,14 @@ __device__ __forceinline__ void mbar_arrive(uint64_t* bar) {
   asm volatile(
       "{\n.reg .b64 st;\n"
       "mbarrier.arrive.shared::cta.b64 st, [%0];\n}\n" ::"r"(smem_u32(bar))
+      : "memory");
+}
+// the same, n arrivals at once
+__device__ __forceinline__ void mbar_arrive_n(uint64_t* bar, uint32_t n) {
+  asm volatile(
+      "{\n.reg .b64 st;\n"
+      "mbarrier.arrive.shared::cta.b64 st, [%0], %1;\n}\n" ::"r"(smem_u32(bar)),
+      "r"(n)
       : "memory");
 }
 __device__ __forceinline__ bool mbar_try_wait(uint64_t* bar, uint32_t parity) {
@@ -118,21 +168,6 @@ __device__ __forceinline__ bool mbar_wait_bounded(uint64_t* bar, uint32_t parity
     if ((it & 63) == 0 && global_ns() - t0 > max_ns) return false;
   }
   return false;
-}
-
-// ------------------------------------------------------------------ cp.async (16 B)
-// asynchronous global -> shared copy of 16 bytes (both 16-byte aligned), L2 only
-__device__ __forceinline__ void cp_async16(void* smem_dst, const void* gsrc) {
-  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(smem_u32(smem_dst)),
-               "l"(gsrc)
-               : "memory");
-}
-__device__ __forceinline__ void cp_async_commit() {
-  asm volatile("cp.async.commit_group;" ::: "memory");
-}
-// waits for all of this thread's committed copies
-__device__ __forceinline__ void cp_async_wait_all() {
-  asm volatile("cp.async.wait_group 0;" ::: "memory");
 }
 
 // ------------------------------------------------------------------ fences
