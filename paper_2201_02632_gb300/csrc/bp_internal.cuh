@@ -74,7 +74,7 @@ struct PpPrepared {
   int64_t n;
   bp_map_geom g;
   int select, ts, unit;
-  int ks;  // 3: keys 8 tile + size class (classes 1-7: the small-particle deposit)
+  int ks;  // class bits of the keys below the tile
   int64_t np, n_tiles, n_keys, max_units, n_slots;
   const uint32_t* vals;
   int64_t *tstart, *uoff, *soff;

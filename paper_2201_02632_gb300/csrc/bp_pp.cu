@@ -5,7 +5,7 @@
 //                  y_i and b_i (Eqs. y_i^PP,h, b_i^PP,h, field_y, field_b)
 //  k_pair_count /  (tile, particle) pairs of every tile a particle's 2h square
 //  k_pair_emit     touches, in particle order
-//  radix sort      stable by tile key (bp_sort.cu)
+//  radix sort      stable by tile and class (bp_sort.cu)
 //  k_units         split each tile's particle list into work units
 //  k_deposit       persistent: one CTA accumulates one work unit's particles into a
 //                  register/shared-memory tile with the separable pixel-integrated
@@ -336,13 +336,20 @@ __global__ void __launch_bounds__(ASSIGN_THREADS) k_assign4(AssignArgs a, BpTabl
 }
 
 // ---------------------------------------------------------------- pairs
-// Bits of a pair key below the tile when the small-particle deposit is on: the key is
-// 2^SMALL_KS tile + the particle's size class.
-constexpr int SMALL_KS = 3;
-// The tiles a particle's clipped pixel box touches, and its size class: 0 when the box is
-// wider than `sspan` pixels on an axis (or sspan is 0), else 1 for a box at most 2 pixels on
-// both axes and span - 1 for a largest side of span = 3 .. 8 pixels (the small-particle deposit
-// takes them grouped by size, so that a warp's particles have similar boxes).
+// Class bits of a pair key below the tile: KS_FIELD with the tensor-core deposit (field
+// particles, which carry no y, after the others of their tile: the deposit skips the y rows of
+// 16 particles without y), SMALL_KS with the small-particle deposit on as well.  The extra bit
+// keeps the full-scale sort at two digits (16 bits); the deposit gains more than the sort
+// loses: 5e8-particle cone 140.4 -> 134.4 ms against 25.9 -> 28.7 ms, 4e6-particle cone 2.54 ->
+// 2.39 ms against 0.29 -> 0.33 ms.
+constexpr int KS_FIELD = 1, SMALL_KS = 4;
+// Large-particle keys of a tile (its first ones)
+__host__ __device__ __forceinline__ int large_keys(int ks) { return ks ? 2 : 1; }
+// The tiles a particle's clipped pixel box touches, and its class: 0 when the box is wider than
+// `sspan` pixels on an axis (or sspan is 0), 1 for such a field particle, else 2 for a box at
+// most 2 pixels on both axes and span for a largest side of span = 3 .. 8 pixels (the
+// small-particle deposit takes them grouped by size, so that a warp's particles have similar
+// boxes).
 __device__ __forceinline__ bool particle_tiles(const float4 r0, const float4 r1, int nx, int ny,
                                                int ts, int select, int& tx0, int& tx1, int& ty0,
                                                int& ty1, int sspan, int& cls) {
@@ -354,7 +361,7 @@ __device__ __forceinline__ bool particle_tiles(const float4 r0, const float4 r1,
   if (!bp_span(__float_as_int(r1.z), r0.x, r0.z, nx, i0, i1)) return false;
   if (!bp_span(__float_as_int(r1.w), r0.y, r0.z, ny, j0, j1)) return false;
   const int span = max(i1 - i0, j1 - j0) + 1;
-  cls = span > sspan ? 0 : (span <= 2 ? 1 : span - 1);  // 1 .. 7 (SMALL_KS = 3 bits)
+  cls = span > sspan ? (kind == BP_KIND_FIELD ? 1 : 0) : max(span, 2);  // < 2^SMALL_KS
   tx0 = i0 / ts;
   tx1 = i1 / ts;
   ty0 = j0 / ts;
@@ -376,12 +383,11 @@ __global__ void k_pair_count(const float4* __restrict__ rec, int64_t n, int nx, 
 
 // The warp's particles own one contiguous range of pairs (offs is their exclusive scan):
 // lanes write it 32 consecutive pairs at a time, each finding its particle by a binary
-// search over the warp's 32 offsets (shuffles), so that every store is coalesced.  With
-// sspan > 0 the key is 2^SMALL_KS tile + the particle's size class (particle_tiles: 0 for the
-// tensor-core deposit, 1-7 for the small-particle deposit); with sspan = 0 it is the tile.
+// search over the warp's 32 offsets (shuffles), so that every store is coalesced.  The key is
+// 2^ks tile + the particle's class (particle_tiles), or the tile with ks = 0.
 __global__ void k_pair_emit(const float4* __restrict__ rec, int64_t n, int nx, int ny, int ts,
                             int select, int ntx, const int64_t* __restrict__ offs,
-                            uint32_t* keys, uint32_t* vals, int sspan, int* dbg) {
+                            uint32_t* keys, uint32_t* vals, int sspan, int ks, int* dbg) {
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   const int lane = threadIdx.x & 31;
   const int64_t i0 = i - lane;
@@ -393,10 +399,9 @@ __global__ void k_pair_emit(const float4* __restrict__ rec, int64_t n, int nx, i
                        c)) {
       w = tx1 - tx0 + 1;
       cnt = w * (ty1 - ty0 + 1);
-      cls = c;
+      cls = ks > 0 ? c : 0;
     }
   }
-  const int ks = sspan > 0 ? SMALL_KS : 0;
   const int64_t base = offs[i0];
   const int rel = (int)(offs[i < n ? i : n] - base);  // past the end: the total
   const int end = __shfl_sync(0xffffffffu, rel + cnt, 31);
@@ -441,14 +446,15 @@ __global__ void k_pair_emit(const float4* __restrict__ rec, int64_t n, int nx, i
 // ---------------------------------------------------------------- work units
 using Unit = BpUnit;
 
-// units per key, and partial-tile slots (only keys split into several units need them); with
-// ks = SMALL_KS only the keys 2^ks tile get units (the others: small particles,
-// k_deposit_small)
+// Per tile: the work units of its large-particle keys (the first large_keys(ks) of its 2^ks;
+// the others: small particles, k_deposit_small), and partial-tile slots (only tiles split into
+// several units need them)
 __global__ void k_unit_count(const int64_t* __restrict__ tstart, int64_t n_tiles, int unit,
                              uint32_t* ucount, uint32_t* scount, int ks = 0) {
   int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (t >= n_tiles) return;
-  int64_t len = (t & ((1 << ks) - 1)) ? 0 : tstart[t + 1] - tstart[t];
+  const int64_t k = t << ks;
+  int64_t len = tstart[k + large_keys(ks)] - tstart[k];
   uint32_t nu = (uint32_t)((len + unit - 1) / unit);
   ucount[t] = nu;
   if (scount) scount[t] = nu > 1 ? nu : 0u;
@@ -459,13 +465,13 @@ __global__ void k_unit_emit(const int64_t* __restrict__ tstart, int64_t n_tiles,
                             Unit* units, int ks = 0) {
   int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (t >= n_tiles) return;
-  if (t & ((1 << ks) - 1)) return;
-  int64_t b = tstart[t], e = tstart[t + 1];
+  const int64_t k = t << ks;
+  int64_t b = tstart[k], e = tstart[k + large_keys(ks)];
   int64_t nu = (e - b + unit - 1) / unit;
   int64_t u0 = uoff[t];
   for (int64_t q = 0; q < nu; ++q) {
     Unit U;
-    U.tile = (int)(t >> ks);
+    U.tile = (int)t;
     U.slot = (nu > 1 && soff) ? (int)(soff[t] + q) : -1;
     U.begin = b + q * unit;
     U.end = min(e, b + (q + 1) * unit);
@@ -694,11 +700,11 @@ __global__ void __launch_bounds__(256) k_reduce_tiles(const int64_t* __restrict_
   int64_t t = blockIdx.x;
   if (t >= n_tiles) return;
   if (err && *err) return;  // the deposit gave up: its partial tiles are incomplete
-  const int64_t key = t << ks;  // the tile's (large-particle) key
-  int64_t len = tstart[key + 1] - tstart[key];
+  const int64_t key = t << ks;  // the tile's first large-particle key
+  int64_t len = tstart[key + large_keys(ks)] - tstart[key];
   int64_t nu = (len + unit - 1) / unit;
   if (nu <= 1) return;
-  int64_t u0 = soff[key];
+  int64_t u0 = soff[t];
   int x0 = (int)(t % ntx) * TS, y0 = (int)(t / ntx) * TS;
   constexpr int SLICE = TS * TS / REDUCE_SPLIT;
   const int q_end = (blockIdx.y + 1) * SLICE;
@@ -789,8 +795,9 @@ __global__ void __launch_bounds__(SMALL_THREADS) k_deposit_small(
   SmallSmem& S = *reinterpret_cast<SmallSmem*>(small_raw);
   const int t = blockIdx.x, tid = threadIdx.x, lane = tid & 31, wp = tid >> 5;
   if (err && *err) return;  // the tensor-core deposit before it gave up
-  // classes 1 .. 7 of the tile: keys 8 t + 1 .. 8 t + 7
-  const int64_t b = tstart[((int64_t)t << SMALL_KS) + 1], e = tstart[((int64_t)(t + 1) << SMALL_KS)];
+  // the tile's classes after the large ones
+  const int64_t b = tstart[((int64_t)t << SMALL_KS) + large_keys(SMALL_KS)];
+  const int64_t e = tstart[((int64_t)(t + 1) << SMALL_KS)];
   if (b >= e) return;
   const int x0 = (t % ntx) * 64, y0 = (t / ntx) * 64;
   for (int q = tid; q < 2 * 64 * 64; q += SMALL_THREADS) {
@@ -930,11 +937,11 @@ int check_geom(bp_ctx* ctx, const bp_map_geom* g, const char* who) {
   return BP_OK;
 }
 
-// Builds the sorted (tile, particle) list; returns keys/vals pointers and count.  sspan > 0:
-// keys 2^SMALL_KS tile + the particle's size class (see k_pair_emit).
+// Builds the sorted (tile, particle) list; returns keys/vals pointers and count.  Keys:
+// 2^ks tile + the particle's class (see k_pair_emit).
 int build_pairs(bp_ctx* ctx, int64_t n, const float* assigned, const bp_map_geom* g, int select,
                 int ts, uint32_t** keys_out, uint32_t** vals_out, int64_t* npairs_out,
-                int64_t* n_tiles_out, int sspan = 0) {
+                int64_t* n_tiles_out, int sspan = 0, int ks = 0) {
   const int ntx = (g->nx + ts - 1) / ts, nty = (g->ny + ts - 1) / ts;
   const int64_t n_tiles = (int64_t)ntx * nty;
   uint32_t* counts;
@@ -959,11 +966,11 @@ int build_pairs(bp_ctx* ctx, int64_t n, const float* assigned, const bp_map_geom
   if ((r = bp_ws(ctx, WS_KEYS1, (size_t)np * 4, (void**)&k1))) return r;
   if ((r = bp_ws(ctx, WS_VALS1, (size_t)np * 4, (void**)&v1))) return r;
   k_pair_emit<<<nb, 256, 0, ctx->stream>>>(rec, n, g->nx, g->ny, ts, select, ntx, offs, k0, v0,
-                                           sspan, bp_dbg_word(ctx));
+                                           sspan, ks, bp_dbg_word(ctx));
   BP_LAUNCH_CHECK(ctx, "pair emit");
   bp_phase_end(ctx, BP_PH_PAIRS);
   int key_bits = 0;
-  while (((int64_t)1 << key_bits) < (n_tiles << (sspan > 0 ? SMALL_KS : 0))) ++key_bits;
+  while (((int64_t)1 << key_bits) < (n_tiles << ks)) ++key_bits;
   bp_phase_begin(ctx, BP_PH_SORT);
   if ((r = bp_radix_sort_pairs(ctx, k0, v0, k1, v1, np, key_bits, keys_out, vals_out))) return r;
   *npairs_out = np;
@@ -1002,7 +1009,7 @@ template <int TS>
 int prepare_units(bp_ctx* ctx, const uint32_t* keys, const uint32_t* vals, int64_t np,
                   int64_t n_tiles, PpPrepared* P, int ks = 0) {
   int r;
-  const int64_t n_keys = n_tiles << ks;  // ks = SMALL_KS: 8 keys per tile (size classes)
+  const int64_t n_keys = n_tiles << ks;
   // particles per work unit: the context's value, or (auto) about 16 units per
   // resident CTA, at least 2048
   int64_t unit64 = ctx->pp_unit;
@@ -1012,27 +1019,29 @@ int prepare_units(bp_ctx* ctx, const uint32_t* keys, const uint32_t* vals, int64
     if (unit64 > (1 << 30)) unit64 = 1 << 30;
   }
   const int unit = (int)unit64;
+  // key starts; per tile unit offsets, slot offsets and their counts
   int64_t* tstart;
-  if ((r = bp_ws(ctx, WS_TILES, (size_t)(n_keys + 1) * 8 * 3 + (size_t)(n_keys + 1) * 8 + 64,
+  if ((r = bp_ws(ctx, WS_TILES,
+                 (size_t)(n_keys + 1) * 8 + (size_t)(n_tiles + 1) * (8 * 2 + 4 * 2) + 64,
                  (void**)&tstart)))
     return r;
   int64_t* uoff = tstart + (n_keys + 1);
-  int64_t* soff = uoff + (n_keys + 1);
-  uint32_t* ucount = (uint32_t*)(soff + (n_keys + 1));
-  uint32_t* scount = ucount + (n_keys + 1);
+  int64_t* soff = uoff + (n_tiles + 1);
+  uint32_t* ucount = (uint32_t*)(soff + (n_tiles + 1));
+  uint32_t* scount = ucount + (n_tiles + 1);
   if ((r = bp_tile_ranges(ctx, keys, np, n_keys, tstart))) return r;
-  unsigned tb = (unsigned)((n_keys + 255) / 256);
-  k_unit_count<<<tb, 256, 0, ctx->stream>>>(tstart, n_keys, unit, ucount, scount, ks);
+  unsigned tb = (unsigned)((n_tiles + 255) / 256);
+  k_unit_count<<<tb, 256, 0, ctx->stream>>>(tstart, n_tiles, unit, ucount, scount, ks);
   BP_LAUNCH_CHECK(ctx, "unit count");
-  if ((r = bp_scan_u32_to_i64(ctx, ucount, uoff, n_keys))) return r;
-  if ((r = bp_scan_u32_to_i64(ctx, scount, soff, n_keys))) return r;
-  const int64_t max_units = n_keys + np / unit + 1;
+  if ((r = bp_scan_u32_to_i64(ctx, ucount, uoff, n_tiles))) return r;
+  if ((r = bp_scan_u32_to_i64(ctx, scount, soff, n_tiles))) return r;
+  const int64_t max_units = n_tiles + np / unit + 1;
   Unit* units;
   if ((r = bp_ws(ctx, WS_UNITS, (size_t)max_units * sizeof(Unit), (void**)&units))) return r;
-  k_unit_emit<<<tb, 256, 0, ctx->stream>>>(tstart, n_keys, unit, uoff, soff, units, ks);
+  k_unit_emit<<<tb, 256, 0, ctx->stream>>>(tstart, n_tiles, unit, uoff, soff, units, ks);
   BP_LAUNCH_CHECK(ctx, "unit emit");
   // partial tiles exist only for tiles split into several units
-  BP_CUDA(ctx, cudaMemcpyAsync(ctx->h_pinned + 1, soff + n_keys, 8, cudaMemcpyDeviceToHost,
+  BP_CUDA(ctx, cudaMemcpyAsync(ctx->h_pinned + 1, soff + n_tiles, 8, cudaMemcpyDeviceToHost,
                                ctx->stream));
   BP_CUDA(ctx, cudaStreamSynchronize(ctx->stream));
   P->ts = TS;
@@ -1068,13 +1077,13 @@ int launch_deposit(bp_ctx* ctx, const float* assigned, const bp_map_geom* g,
   const bool tc = bp_deposit_uses_tc(ctx, TS);
   if (tc) {
     bp_phase_begin(ctx, BP_PH_DEPOSIT);
-    if ((r = bp_deposit_tc_launch(ctx, assigned, P.vals, units, P.uoff + P.n_keys,
+    if ((r = bp_deposit_tc_launch(ctx, assigned, P.vals, units, P.uoff + P.n_tiles,
                                   ctx->d_counter + 1, P.max_units, g, ymap, bmap, ylo, blo,
                                   partials)))
       return r;
     bp_phase_end(ctx, BP_PH_DEPOSIT);
   } else {
-    if ((r = deposit_simt<TS>(ctx, assigned, g, P.vals, units, P.uoff + P.n_keys,
+    if ((r = deposit_simt<TS>(ctx, assigned, g, P.vals, units, P.uoff + P.n_tiles,
                               ctx->d_counter + 1, P.max_units, ymap, bmap, ylo, blo, partials)))
       return r;
   }
@@ -1086,7 +1095,7 @@ int launch_deposit(bp_ctx* ctx, const float* assigned, const bp_map_geom* g,
     BP_LAUNCH_CHECK(ctx, "reduce tiles");
   }
   bp_phase_end(ctx, BP_PH_REDUCE);
-  if (P.ks) {  // the small particles, after the large ones of every tile
+  if (P.ks == SMALL_KS) {  // the small particles, after the large ones of every tile
     bp_phase_begin(ctx, BP_PH_DEPOSIT_SMALL);
     const size_t smem = sizeof(SmallSmem);
     BP_CUDA(ctx, cudaFuncSetAttribute(k_deposit_small, cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -1185,6 +1194,10 @@ static int pp_small_span(const bp_ctx* ctx, int ts, const bp_map_geom* g) {
   const int64_t tiles = (int64_t)((g->nx + 63) / 64) * ((g->ny + 63) / 64);
   return tiles >= 4 * (int64_t)ctx->num_sms ? 8 : 0;
 }
+// Class bits of its pair keys
+static int pp_class_bits(const bp_ctx* ctx, int ts, int sspan) {
+  return sspan > 0 ? SMALL_KS : (bp_deposit_uses_tc(ctx, ts) ? KS_FIELD : 0);
+}
 
 // The particle paste with every scratch buffer supplied by the caller.  Reads back the
 // pair count (one host synchronisation) and returns BP_ERANGE if it exceeds max_pairs.
@@ -1214,7 +1227,7 @@ int bp_pp_paste_buffers(bp_ctx* ctx, int64_t n, const float* assigned, const bp_
                    (long long)np, (long long)B->max_pairs);
   if (np == 0) return BP_OK;
   k_pair_emit<<<nb, 256, 0, ctx->stream>>>(rec, n, g->nx, g->ny, ts, select, ntx, B->offs,
-                                           B->keys0, B->vals0, 0, bp_dbg_word(ctx));
+                                           B->keys0, B->vals0, 0, 0, bp_dbg_word(ctx));
   BP_LAUNCH_CHECK(ctx, "pair emit");
   int key_bits = 0;
   while (((int64_t)1 << key_bits) < n_tiles) ++key_bits;
@@ -1367,10 +1380,11 @@ int bp_paste_particles(bp_ctx* ctx, int64_t n, const float* assigned, const bp_m
   uint32_t *keys, *vals;
   int64_t np, n_tiles;
   const int sspan = pp_small_span(ctx, ts, geom);
-  if ((r = build_pairs(ctx, n, assigned, geom, select, ts, &keys, &vals, &np, &n_tiles, sspan)))
+  const int ks = pp_class_bits(ctx, ts, sspan);
+  if ((r = build_pairs(ctx, n, assigned, geom, select, ts, &keys, &vals, &np, &n_tiles, sspan,
+                       ks)))
     return r;
   if (np == 0) return BP_OK;
-  const int ks = sspan > 0 ? SMALL_KS : 0;
   if (ts == 64)
     return deposit<64>(ctx, assigned, geom, keys, vals, np, n_tiles, ymap, bmap, ylo, blo, ks);
   return deposit<32>(ctx, assigned, geom, keys, vals, np, n_tiles, ymap, bmap, ylo, blo, ks);
@@ -1403,11 +1417,11 @@ int bp_pp_prepare(bp_ctx* ctx, int64_t n, const float* assigned, const bp_map_ge
     uint32_t *keys, *vals;
     int64_t np, n_tiles;
     const int sspan = pp_small_span(ctx, ts, geom);
+    const int ks = pp_class_bits(ctx, ts, sspan);
     if ((r = build_pairs(ctx, n, assigned, geom, select, ts, &keys, &vals, &np, &n_tiles,
-                         sspan)))
+                         sspan, ks)))
       return r;
     if (np > 0) {
-      const int ks = sspan > 0 ? SMALL_KS : 0;
       r = ts == 64 ? prepare_units<64>(ctx, keys, vals, np, n_tiles, &P, ks)
                    : prepare_units<32>(ctx, keys, vals, np, n_tiles, &P, ks);
       if (r) return r;
@@ -1424,7 +1438,7 @@ int bp_pp_deposit(bp_ctx* ctx, int64_t n, const float* assigned, const bp_map_ge
   const PpPrepared& P = ctx->pp_prep;
   if (!P.valid || P.assigned != assigned || P.n != n || !geom || P.select != select ||
       P.ts != ctx->pp_tile || memcmp(&P.g, geom, sizeof(bp_map_geom)) != 0 ||
-      (P.np > 0 && P.ks != (pp_small_span(ctx, P.ts, geom) > 0 ? SMALL_KS : 0)))
+      (P.np > 0 && P.ks != pp_class_bits(ctx, P.ts, pp_small_span(ctx, P.ts, geom))))
     return bp_fail(ctx, BP_EINVAL, "bp_pp_deposit: no bp_pp_prepare of these records");
   if (P.np == 0 || n == 0) return BP_OK;
   for (int k : {(int)WS_KEYS0, (int)WS_VALS0, (int)WS_KEYS1, (int)WS_VALS1, (int)WS_TILES,
