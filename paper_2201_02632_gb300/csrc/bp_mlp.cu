@@ -4,10 +4,9 @@
 // features (log10 M, log10 c, z, eps_*, f_*, eps_DM; normalised) to the solved model
 // (ln r_f/r_vir, ln T r_vir/(G M), ln rho0/rho_s; normalised).
 //
-//  training (FP32):  k_dense (forward layer, bias + GELU epilogue), k_dense with the
-//                    transposed weight (data gradient, GELU' epilogue), k_wgrad (per
-//                    row-chunk weight/bias gradient partials) + k_sum_partials (fixed
-//                    order), k_adam
+//  training (FP32):  k_forward (all four layers of a tile of rows), k_backward (data and
+//                    weight gradients of a tile, all layers; one set of weight-gradient
+//                    partials per CTA) + k_sum_partials (fixed order), k_adam
 //  inference:        k_infer_tc, all four layers fused per 128-row tile, BF16 weights and
 //                    activations, FP32 accumulation; the two 128 x 128 layers on the
 //                    tensor cores (tcgen05, accumulator in tensor memory)
@@ -17,6 +16,7 @@
 // rejected halos get the full solve).
 #include <cuda_bf16.h>
 
+#include <algorithm>
 #include <vector>
 
 #include "bp_internal.cuh"
@@ -47,163 +47,334 @@ __device__ __forceinline__ float gelu_grad(float x) {
   return cdf + x * pdf;
 }
 
-constexpr int ROWS = 64;  // rows per CTA of the dense kernels
-constexpr int DT = 256;
+// ---------------------------------------------------------------- FP32 training kernels
+// One CTA of 8 warps per SM, persistent over tiles of 32 rows, with W2 and W3 in shared memory
+// ([out][in], rows padded to 132 floats: the lanes' 16-byte reads hit all banks whether they
+// run over outputs or inputs).  Warp w owns rows 4 w .. 4 w + 3 of the tile through every layer,
+// so the layers need no CTA barrier; a lane computes 4 rows x 4 outputs (or inputs) and reads 8
+// 16-byte words of shared memory per 64 multiply-adds: the kernels are bound by shared-memory
+// reads (5 wavefronts per 16 multiply-add instructions), and by latency at one tile per SM.
+// Measured at 4096 rows (one training step of 17 launches took 398 us: the weight gradients ran
+// on 16 CTAs, each layer was a launch, and every activation went through global memory twice):
+// k_forward 20 us (68 us as four launches), k_backward + k_sum_partials 40 us (296 us as
+// 13 launches).  32 rows per tile puts 128 tiles on 152 SMs at the training batch of 4096.
+constexpr int MT_ROWS = 32, MT_THREADS = 256;
+constexpr int LDW = HID + 4;  // padded row length in shared memory
 
-// C[r][o] = sum_i X[r][i] W'[o][i] (+ bias, activation epilogue), for OUT_N <= 128 outputs
-// and IN_K inputs, inputs staged in chunks of KC.  W' is W ([OUT_N][IN_K], forward) or
-// W^T (TRANS: W is [IN_K][OUT_N], data gradient).  EPI 0: C = acc + b;
-// 1: Z = acc + b, A = GELU(Z); 2: C = acc * GELU'(Zp)
-constexpr int KC = 32;
-template <int IN_K, int OUT_N, bool TRANS, int EPI>
-__global__ void __launch_bounds__(DT) k_dense(int64_t n, const float* __restrict__ X,
-                                              int ldx, const float* __restrict__ W,
-                                              const float* __restrict__ b,
-                                              const float* __restrict__ Zp, int ldzp,
-                                              float* __restrict__ C, int ldc,
-                                              float* __restrict__ A2, int lda2) {
-  constexpr int OPAD = (OUT_N + 3) / 4 * 4;
-  static_assert(OPAD <= 128, "at most 128 outputs");
-  __shared__ __align__(16) float Xs[KC][ROWS + 4];
-  __shared__ __align__(16) float Ws[KC][OPAD + 4];
-  const int tid = threadIdx.x, w = tid >> 5, lane = tid & 31;
-  const int64_t row0 = (int64_t)blockIdx.x * ROWS;
-  const int o0 = lane * 4;  // this lane's four outputs (valid while o0 < OPAD)
-  float acc[8][4];
-#pragma unroll
-  for (int r = 0; r < 8; ++r)
-#pragma unroll
-    for (int c = 0; c < 4; ++c) acc[r][c] = 0.f;
-  for (int k0 = 0; k0 < IN_K; k0 += KC) {
-    const int kn = min(KC, IN_K - k0);
-    __syncthreads();
-    for (int idx = tid; idx < kn * OPAD; idx += DT) {
-      int o = idx % OPAD, i = idx / OPAD;
-      float v = 0.f;
-      if (o < OUT_N) v = TRANS ? W[(int64_t)(k0 + i) * OUT_N + o] : W[(int64_t)o * IN_K + k0 + i];
-      Ws[i][o] = v;
-    }
-    for (int idx = tid; idx < ROWS * kn; idx += DT) {
-      int r = idx / kn, i = idx % kn;
-      int64_t row = row0 + r;
-      Xs[i][r] = row < n ? X[row * ldx + k0 + i] : 0.f;
-    }
-    __syncthreads();
-    if (o0 < OPAD) {
-      for (int i = 0; i < kn; ++i) {
-        float4 xa = *reinterpret_cast<const float4*>(&Xs[i][w * 8]);
-        float4 xb = *reinterpret_cast<const float4*>(&Xs[i][w * 8 + 4]);
-        float4 wv = *reinterpret_cast<const float4*>(&Ws[i][o0]);
-        float xr[8] = {xa.x, xa.y, xa.z, xa.w, xb.x, xb.y, xb.z, xb.w};
-        float wc[4] = {wv.x, wv.y, wv.z, wv.w};
-#pragma unroll
-        for (int r = 0; r < 8; ++r)
-#pragma unroll
-          for (int c = 0; c < 4; ++c) acc[r][c] = fmaf(xr[r], wc[c], acc[r][c]);
-      }
-    }
-  }
-  if (o0 >= OPAD) return;
-#pragma unroll
-  for (int r = 0; r < 8; ++r) {
-    int64_t row = row0 + w * 8 + r;
-    if (row >= n) continue;
-#pragma unroll
-    for (int c = 0; c < 4; ++c) {
-      int o = o0 + c;
-      if (o >= OUT_N) continue;
-      float v = acc[r][c];
-      if (EPI == 0) {
-        C[row * ldc + o] = v + b[o];
-      } else if (EPI == 1) {
-        float z = v + b[o];
-        C[row * ldc + o] = z;
-        A2[row * lda2 + o] = gelu(z);
-      } else {
-        C[row * ldc + o] = v * gelu_grad(Zp[row * ldzp + o]);
-      }
-    }
-  }
-}
+struct MtForward {
+  float w2[HID][LDW], w3[HID][LDW];
+  float a[2][MT_ROWS][LDW];  // activations of the layer before and of this one
+  float w1[HID][IN], w4[OUT][HID];
+  float b1[HID], b2[HID], b3[HID], b4[4];
+};
+struct MtBackward {
+  float w2[HID][LDW], w3[HID][LDW];
+  float d[3][MT_ROWS][LDW];  // gradients of the pre-activations of layers 3, 2, 1
+  float a[MT_ROWS][LDW];     // activations the weight gradient takes
+  float x[MT_ROWS][8], dy[MT_ROWS][4];
+  float w4[OUT][HID];
+};
 
-// Weight-gradient partials: for the rows of chunk blockIdx.x,
-// P[chunk][o * IN_K + i] = sum_r D[r][o] Xp[r][i] and P[chunk][OUT_N * IN_K + o] = sum_r D[r][o]
-constexpr int WG_ROWS = 256;
-template <int IN_K, int OUT_N>
-__global__ void __launch_bounds__(DT) k_wgrad(int64_t n, const float* __restrict__ D, int ldd,
-                                              const float* __restrict__ Xp, int ldx,
-                                              float* __restrict__ P) {
-  constexpr int NO = OUT_N * IN_K + OUT_N;
-  const int64_t r0 = (int64_t)blockIdx.x * WG_ROWS;
-  const int64_t r1 = min(n, r0 + WG_ROWS);
-  float* out = P + (int64_t)blockIdx.x * NO;
-  if (IN_K == HID && OUT_N == HID) {
-    // register-tiled: thread owns 8 outputs o x 8 inputs i
-    __shared__ __align__(16) float Ds[32][HID];
-    __shared__ __align__(16) float As[32][HID];
-    const int tid = threadIdx.x;
-    const int og = (tid >> 4) * 8, ig = (tid & 15) * 8;
-    float acc[8][8];
-    float bacc[8];
-#pragma unroll
-    for (int a = 0; a < 8; ++a) {
-      bacc[a] = 0.f;
-#pragma unroll
-      for (int c = 0; c < 8; ++c) acc[a][c] = 0.f;
-    }
-    for (int64_t rb = r0; rb < r1; rb += 32) {
-      __syncthreads();
-      for (int idx = tid; idx < 32 * HID; idx += DT) {
-        int r = idx / HID, c = idx % HID;
-        int64_t row = rb + r;
-        Ds[r][c] = row < r1 ? D[row * ldd + c] : 0.f;
-        As[r][c] = row < r1 ? Xp[row * ldx + c] : 0.f;
-      }
-      __syncthreads();
-      for (int r = 0; r < 32; ++r) {
-        float4 d0 = *reinterpret_cast<const float4*>(&Ds[r][og]);
-        float4 d1 = *reinterpret_cast<const float4*>(&Ds[r][og + 4]);
-        float4 a0 = *reinterpret_cast<const float4*>(&As[r][ig]);
-        float4 a1 = *reinterpret_cast<const float4*>(&As[r][ig + 4]);
-        float dv[8] = {d0.x, d0.y, d0.z, d0.w, d1.x, d1.y, d1.z, d1.w};
-        float av[8] = {a0.x, a0.y, a0.z, a0.w, a1.x, a1.y, a1.z, a1.w};
-#pragma unroll
-        for (int a = 0; a < 8; ++a) {
-          bacc[a] += dv[a];
-#pragma unroll
-          for (int c = 0; c < 8; ++c) acc[a][c] = fmaf(dv[a], av[c], acc[a][c]);
-        }
-      }
-    }
-#pragma unroll
-    for (int a = 0; a < 8; ++a) {
-#pragma unroll
-      for (int c = 0; c < 8; ++c) out[(og + a) * IN_K + ig + c] = acc[a][c];
-      if ((tid & 15) == 0) out[OUT_N * IN_K + og + a] = bacc[a];
-    }
+// a [HID][HID] matrix into padded shared rows (16-byte loads when src allows them)
+__device__ __forceinline__ void mt_load_w(float (*dst)[LDW], const float* __restrict__ src) {
+  if ((reinterpret_cast<uintptr_t>(src) & 15) == 0) {
+    for (int q = threadIdx.x; q < HID * HID / 4; q += MT_THREADS)
+      *reinterpret_cast<float4*>(&dst[q >> 5][4 * (q & 31)]) =
+          __ldg(reinterpret_cast<const float4*>(src) + q);
   } else {
-    for (int j = threadIdx.x; j < NO; j += DT) {
-      float acc = 0.f;
-      if (j < OUT_N * IN_K) {
-        int o = j / IN_K, i = j % IN_K;
-        for (int64_t r = r0; r < r1; ++r) acc = fmaf(D[r * ldd + o], Xp[r * ldx + i], acc);
-      } else {
-        int o = j - OUT_N * IN_K;
-        for (int64_t r = r0; r < r1; ++r) acc += D[r * ldd + o];
+    for (int q = threadIdx.x; q < HID * HID; q += MT_THREADS) dst[q >> 7][q & 127] = src[q];
+  }
+}
+
+// acc[r][j] += sum_k in[r][k] w[lane + 32 j][k] for the warp's four rows
+__device__ __forceinline__ void mt_gemm_nt(const float (*in)[LDW], const float (*w)[LDW], int lane,
+                                           float (&acc)[4][4]) {
+#pragma unroll 4
+  for (int k = 0; k < HID; k += 4) {
+    float4 xv[4], wv[4];
+#pragma unroll
+    for (int r = 0; r < 4; ++r) xv[r] = *reinterpret_cast<const float4*>(&in[r][k]);
+#pragma unroll
+    for (int j = 0; j < 4; ++j) wv[j] = *reinterpret_cast<const float4*>(&w[lane + 32 * j][k]);
+#pragma unroll
+    for (int r = 0; r < 4; ++r)
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        acc[r][j] = fmaf(xv[r].x, wv[j].x, acc[r][j]);
+        acc[r][j] = fmaf(xv[r].y, wv[j].y, acc[r][j]);
+        acc[r][j] = fmaf(xv[r].z, wv[j].z, acc[r][j]);
+        acc[r][j] = fmaf(xv[r].w, wv[j].w, acc[r][j]);
       }
-      out[j] = acc;
+  }
+}
+
+// acc[r][j] += sum_o d[r][o] w[o][4 lane + j] for the warp's four rows
+__device__ __forceinline__ void mt_gemm_nn(const float (*d)[LDW], const float (*w)[LDW], int lane,
+                                           float (&acc)[4][4]) {
+#pragma unroll 2
+  for (int o = 0; o < HID; o += 4) {
+    float dv[4][4];
+#pragma unroll
+    for (int r = 0; r < 4; ++r)
+      *reinterpret_cast<float4*>(dv[r]) = *reinterpret_cast<const float4*>(&d[r][o]);
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      const float4 wv = *reinterpret_cast<const float4*>(&w[o + q][4 * lane]);
+#pragma unroll
+      for (int r = 0; r < 4; ++r) {
+        acc[r][0] = fmaf(dv[r][q], wv.x, acc[r][0]);
+        acc[r][1] = fmaf(dv[r][q], wv.y, acc[r][1]);
+        acc[r][2] = fmaf(dv[r][q], wv.z, acc[r][2]);
+        acc[r][3] = fmaf(dv[r][q], wv.w, acc[r][3]);
+      }
     }
   }
 }
 
-// grad[off_w + j] / grad[off_b + o] = sum over chunks, in chunk order
-__global__ void k_sum_partials(const float* __restrict__ P, int64_t nchunks, int nw, int nb,
-                               float* __restrict__ gw, float* __restrict__ gb) {
-  int j = blockIdx.x * blockDim.x + threadIdx.x;
-  if (j >= nw + nb) return;
-  float s = 0.f;
-  for (int64_t c = 0; c < nchunks; ++c) s += P[c * (nw + nb) + j];
-  if (j < nw) gw[j] = s; else gb[j - nw] = s;
+__global__ void __launch_bounds__(MT_THREADS, 1)
+    k_forward(int64_t n, const float* __restrict__ X, const float* __restrict__ par,
+              float* __restrict__ Y, float* __restrict__ cache) {
+  extern __shared__ __align__(16) unsigned char mt_raw[];
+  MtForward& S = *reinterpret_cast<MtForward*>(mt_raw);
+  const int tid = threadIdx.x, w = tid >> 5, lane = tid & 31;
+  constexpr int LC = BP_MLP_CACHE_PER_ROW;
+  mt_load_w(S.w2, par + OFF_W2);
+  mt_load_w(S.w3, par + OFF_W3);
+  for (int q = tid; q < HID * IN; q += MT_THREADS) (&S.w1[0][0])[q] = par[OFF_W1 + q];
+  for (int q = tid; q < OUT * HID; q += MT_THREADS) (&S.w4[0][0])[q] = par[OFF_W4 + q];
+  for (int q = tid; q < HID; q += MT_THREADS) {
+    S.b1[q] = par[OFF_B1 + q];
+    S.b2[q] = par[OFF_B2 + q];
+    S.b3[q] = par[OFF_B3 + q];
+  }
+  if (tid < OUT) S.b4[tid] = par[OFF_B4 + tid];
+  __syncthreads();
+  for (int64_t t = blockIdx.x; t * MT_ROWS < n; t += gridDim.x) {
+    const int64_t row0 = t * MT_ROWS + 4 * w;  // this warp's first row
+    float acc[4][4];
+    // pre-activation + bias and activation of one layer: to the cache and the next layer
+    auto emit = [&](const float* b, int cz, int ca, float (*out)[LDW]) {
+#pragma unroll
+      for (int r = 0; r < 4; ++r)
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+          const int o = lane + 32 * j;
+          const float z = acc[r][j] + b[o], av = gelu(z);
+          if (row0 + r < n) {
+            cache[(row0 + r) * LC + cz + o] = z;
+            cache[(row0 + r) * LC + ca + o] = av;
+          }
+          out[r][o] = av;
+        }
+      __syncwarp();
+    };
+    float(*a0)[LDW] = &S.a[0][4 * w];
+    float(*a1)[LDW] = &S.a[1][4 * w];
+#pragma unroll
+    for (int r = 0; r < 4; ++r) {
+      float x[IN];
+#pragma unroll
+      for (int i = 0; i < IN; ++i) x[i] = row0 + r < n ? X[(row0 + r) * IN + i] : 0.f;
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        float v = 0.f;
+#pragma unroll
+        for (int i = 0; i < IN; ++i) v = fmaf(x[i], S.w1[lane + 32 * j][i], v);
+        acc[r][j] = v;
+      }
+    }
+    emit(S.b1, CZ1, CA1, a0);
+    auto clear = [&]() {
+#pragma unroll
+      for (int r = 0; r < 4; ++r)
+#pragma unroll
+        for (int j = 0; j < 4; ++j) acc[r][j] = 0.f;
+    };
+    clear();
+    mt_gemm_nt(a0, S.w2, lane, acc);
+    emit(S.b2, CZ2, CA2, a1);
+    clear();
+    mt_gemm_nt(a1, S.w3, lane, acc);
+    emit(S.b3, CZ3, CA3, a0);
+    // layer 4: lanes over the inputs, a fixed shuffle tree over the lanes
+#pragma unroll
+    for (int r = 0; r < 4; ++r)
+#pragma unroll
+      for (int o = 0; o < OUT; ++o) {
+        float v = 0.f;
+#pragma unroll
+        for (int j = 0; j < 4; ++j) v = fmaf(a0[r][lane + 32 * j], S.w4[o][lane + 32 * j], v);
+#pragma unroll
+        for (int q = 16; q > 0; q >>= 1) v += __shfl_xor_sync(0xffffffffu, v, q);
+        if (lane == 0 && row0 + r < n) Y[(row0 + r) * OUT + o] = v + S.b4[o];
+      }
+    __syncwarp();
+  }
+}
+
+// The weight gradient of a 128 x 128 layer over the tile's rows: thread (og, ig) owns outputs
+// 4 og + {0..3}, 64 + 4 og + {0..3} and the same of the inputs
+__device__ __forceinline__ void mt_wgrad(const float (*d)[LDW], const float (*a)[LDW], int og,
+                                         int ig, float (&acc)[8][8]) {
+#pragma unroll 2
+  for (int r = 0; r < MT_ROWS; ++r) {
+    float dv[8], av[8];
+    *reinterpret_cast<float4*>(dv) = *reinterpret_cast<const float4*>(&d[r][4 * og]);
+    *reinterpret_cast<float4*>(dv + 4) = *reinterpret_cast<const float4*>(&d[r][64 + 4 * og]);
+    *reinterpret_cast<float4*>(av) = *reinterpret_cast<const float4*>(&a[r][4 * ig]);
+    *reinterpret_cast<float4*>(av + 4) = *reinterpret_cast<const float4*>(&a[r][64 + 4 * ig]);
+#pragma unroll
+    for (int p = 0; p < 8; ++p)
+#pragma unroll
+      for (int q = 0; q < 8; ++q) acc[p][q] = fmaf(dv[p], av[q], acc[p][q]);
+  }
+}
+
+__global__ void __launch_bounds__(MT_THREADS, 1)
+    k_backward(int64_t n, const float* __restrict__ X, const float* __restrict__ par,
+               const float* __restrict__ cache, const float* __restrict__ dY,
+               float* __restrict__ P) {
+  extern __shared__ __align__(16) unsigned char mt_raw[];
+  MtBackward& S = *reinterpret_cast<MtBackward*>(mt_raw);
+  const int tid = threadIdx.x, w = tid >> 5, lane = tid & 31;
+  const int og = tid >> 4, ig = tid & 15;
+  const int c = tid & (HID - 1), half = tid >> 7;  // column and half of the small gradients
+  constexpr int LC = BP_MLP_CACHE_PER_ROW;
+  mt_load_w(S.w2, par + OFF_W2);
+  mt_load_w(S.w3, par + OFF_W3);
+  for (int q = tid; q < OUT * HID; q += MT_THREADS) (&S.w4[0][0])[q] = par[OFF_W4 + q];
+  float g3[8][8], g2[8][8];  // this thread's part of dW3 and dW2
+#pragma unroll
+  for (int p = 0; p < 8; ++p)
+#pragma unroll
+    for (int q = 0; q < 8; ++q) g3[p][q] = g2[p][q] = 0.f;
+  // dW1 (inputs 3 half ..), dW4 (outputs 0, 1 of half 0, output 2 of half 1), biases: half 0
+  // holds db3 and db1 of column c, half 1 db2 and (threads 128 ..) db4
+  float g1[3] = {0.f, 0.f, 0.f}, g4[2] = {0.f, 0.f}, gb[2] = {0.f, 0.f};
+  for (int64_t t = blockIdx.x; t * MT_ROWS < n; t += gridDim.x) {
+    const int64_t base = t * MT_ROWS;
+    const int64_t row0 = base + 4 * w;
+    __syncthreads();  // the tile before is done with the shared arrays
+    for (int q = tid; q < MT_ROWS * 8; q += MT_THREADS) {
+      const int r = q >> 3, i = q & 7;
+      S.x[r][i] = (i < IN && base + r < n) ? X[(base + r) * IN + i] : 0.f;
+      if (i < 4) S.dy[r][i] = (i < OUT && base + r < n) ? dY[(base + r) * OUT + i] : 0.f;
+    }
+    // rows of cached activations, and of pre-activations' GELU' (zeros past the end)
+    auto load_a = [&](int ca) {
+#pragma unroll
+      for (int r = 0; r < 4; ++r)
+#pragma unroll
+        for (int j = 0; j < 4; ++j)
+          S.a[4 * w + r][lane + 32 * j] =
+              row0 + r < n ? cache[(row0 + r) * LC + ca + lane + 32 * j] : 0.f;
+    };
+    float z[4][4];  // pre-activations of columns 4 lane + j
+    auto load_z = [&](int cz) {
+#pragma unroll
+      for (int r = 0; r < 4; ++r)
+#pragma unroll
+        for (int j = 0; j < 4; ++j)
+          z[r][j] = row0 + r < n ? cache[(row0 + r) * LC + cz + 4 * lane + j] : 0.f;
+    };
+    load_a(CA3);
+    load_z(CZ3);
+    __syncthreads();
+    // layer 4 back to the pre-activations of layer 3
+#pragma unroll
+    for (int r = 0; r < 4; ++r)
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        float v = 0.f;
+#pragma unroll
+        for (int o = 0; o < OUT; ++o) v = fmaf(S.dy[4 * w + r][o], S.w4[o][4 * lane + j], v);
+        S.d[0][4 * w + r][4 * lane + j] = v * gelu_grad(z[r][j]);
+      }
+    // dW4, db4
+    for (int r = 0; r < MT_ROWS; ++r) {
+      const float av = S.a[r][c];
+      g4[0] = fmaf(S.dy[r][2 * half], av, g4[0]);
+      if (half == 0) g4[1] = fmaf(S.dy[r][1], av, g4[1]);
+      else if (c < OUT) gb[1] += S.dy[r][c];
+    }
+    load_z(CZ2);
+    __syncthreads();
+    load_a(CA2);
+    float acc[4][4];
+    auto back = [&](int l, const float (*wt)[LDW]) {  // layer 3 - l to the pre-activations before
+#pragma unroll
+      for (int r = 0; r < 4; ++r)
+#pragma unroll
+        for (int j = 0; j < 4; ++j) acc[r][j] = 0.f;
+      mt_gemm_nn(&S.d[l][4 * w], wt, lane, acc);
+#pragma unroll
+      for (int r = 0; r < 4; ++r) {
+        float4 v;
+        v.x = acc[r][0] * gelu_grad(z[r][0]);
+        v.y = acc[r][1] * gelu_grad(z[r][1]);
+        v.z = acc[r][2] * gelu_grad(z[r][2]);
+        v.w = acc[r][3] * gelu_grad(z[r][3]);
+        *reinterpret_cast<float4*>(&S.d[l + 1][4 * w + r][4 * lane]) = v;
+      }
+    };
+    back(0, S.w3);
+    load_z(CZ1);
+    __syncthreads();
+    mt_wgrad(S.d[0], S.a, og, ig, g3);
+    for (int r = 0; r < MT_ROWS; ++r) gb[0] += S.d[half][r][c];  // db3, db2
+    back(1, S.w2);
+    __syncthreads();
+    load_a(CA1);
+    __syncthreads();
+    mt_wgrad(S.d[1], S.a, og, ig, g2);
+    for (int r = 0; r < MT_ROWS; ++r) {
+      const float dv = S.d[2][r][c];
+#pragma unroll
+      for (int i = 0; i < 3; ++i) g1[i] = fmaf(dv, S.x[r][3 * half + i], g1[i]);
+      if (half == 0) gb[1] += dv;  // db1
+    }
+  }
+  float* out = P + (int64_t)blockIdx.x * NPAR;
+#pragma unroll
+  for (int p = 0; p < 8; ++p) {
+    const int o = (p < 4 ? 0 : 60) + 4 * og + p;
+#pragma unroll
+    for (int q = 0; q < 8; ++q) {
+      const int i = (q < 4 ? 0 : 60) + 4 * ig + q;
+      out[OFF_W3 + o * HID + i] = g3[p][q];
+      out[OFF_W2 + o * HID + i] = g2[p][q];
+    }
+  }
+#pragma unroll
+  for (int i = 0; i < 3; ++i) out[OFF_W1 + c * IN + 3 * half + i] = g1[i];
+  out[OFF_W4 + 2 * half * HID + c] = g4[0];
+  if (half == 0) {
+    out[OFF_W4 + HID + c] = g4[1];
+    out[OFF_B3 + c] = gb[0];
+    out[OFF_B1 + c] = gb[1];
+  } else {
+    out[OFF_B2 + c] = gb[0];
+    if (c < OUT) out[OFF_B4 + c] = gb[1];
+  }
+}
+
+// grad[j] = the sum of the CTAs' partials: four threads per parameter, each a contiguous range
+// of the CTAs in order, then their sums in a fixed tree
+constexpr int SP_THREADS = 256, SP_COLS = SP_THREADS / 4;
+__global__ void __launch_bounds__(SP_THREADS)
+    k_sum_partials(const float* __restrict__ P, int ncta, float* __restrict__ grad) {
+  __shared__ float s[4][SP_COLS];
+  const int col = threadIdx.x % SP_COLS, q = threadIdx.x / SP_COLS;
+  const int j = blockIdx.x * SP_COLS + col;
+  const int per = (ncta + 3) / 4, c0 = q * per, c1 = min(ncta, c0 + per);
+  float v = 0.f;
+  if (j < NPAR) {
+#pragma unroll 8
+    for (int k = c0; k < c1; ++k) v += P[(int64_t)k * NPAR + j];
+  }
+  s[q][col] = v;
+  __syncthreads();
+  if (q == 0 && j < NPAR) grad[j] = (s[0][col] + s[1][col]) + (s[2][col] + s[3][col]);
 }
 
 __global__ void k_adam(int np, float* __restrict__ p, const float* __restrict__ g,
@@ -514,6 +685,11 @@ __global__ void k_decode_guess(int64_t n, const float* __restrict__ Y,
   guess[n + i] = g1;
 }
 
+// CTAs of the training kernels: one per tile of rows, at most one per SM
+unsigned mt_grid(const bp_ctx* ctx, int64_t n) {
+  return (unsigned)std::min<int64_t>((n + MT_ROWS - 1) / MT_ROWS, ctx->num_sms);
+}
+
 int check_n(bp_ctx* ctx, int64_t n, const char* who) {
   if (n < 0) return bp_fail(ctx, BP_EINVAL, "%s: n < 0", who);
   if (n > (int64_t)1 << 31) return bp_fail(ctx, BP_ERANGE, "%s: n above 2^31", who);
@@ -530,23 +706,11 @@ int bp_mlp_forward(bp_ctx* ctx, int64_t n, const float* params, const float* x, 
   int r = check_n(ctx, n, "bp_mlp_forward");
   if (r || n == 0) return r;
   if (!params || !x || !y || !cache) return bp_fail(ctx, BP_EINVAL, "bp_mlp_forward: null pointer");
-  unsigned g = (unsigned)((n + ROWS - 1) / ROWS);
-  const int LC = BP_MLP_CACHE_PER_ROW;
-  k_dense<IN, HID, false, 1><<<g, DT, 0, ctx->stream>>>(n, x, IN, params + OFF_W1, params + OFF_B1,
-                                                        nullptr, 0, cache + CZ1, LC, cache + CA1, LC);
-  BP_LAUNCH_CHECK(ctx, "mlp layer 1");
-  k_dense<HID, HID, false, 1><<<g, DT, 0, ctx->stream>>>(n, cache + CA1, LC, params + OFF_W2,
-                                                         params + OFF_B2, nullptr, 0, cache + CZ2,
-                                                         LC, cache + CA2, LC);
-  BP_LAUNCH_CHECK(ctx, "mlp layer 2");
-  k_dense<HID, HID, false, 1><<<g, DT, 0, ctx->stream>>>(n, cache + CA2, LC, params + OFF_W3,
-                                                         params + OFF_B3, nullptr, 0, cache + CZ3,
-                                                         LC, cache + CA3, LC);
-  BP_LAUNCH_CHECK(ctx, "mlp layer 3");
-  k_dense<HID, OUT, false, 0><<<g, DT, 0, ctx->stream>>>(n, cache + CA3, LC, params + OFF_W4,
-                                                         params + OFF_B4, nullptr, 0, y, OUT,
-                                                         nullptr, 0);
-  BP_LAUNCH_CHECK(ctx, "mlp layer 4");
+  BP_CUDA(ctx, cudaFuncSetAttribute(k_forward, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                    (int)sizeof(MtForward)));
+  k_forward<<<mt_grid(ctx, n), MT_THREADS, sizeof(MtForward), ctx->stream>>>(n, x, params, y,
+                                                                            cache);
+  BP_LAUNCH_CHECK(ctx, "mlp forward");
   return BP_OK;
 }
 
@@ -561,52 +725,16 @@ int bp_mlp_backward(bp_ctx* ctx, int64_t n, const float* params, const float* x,
     BP_CUDA(ctx, cudaMemsetAsync(grad, 0, NPAR * sizeof(float), ctx->stream));
     return BP_OK;
   }
-  const int LC = BP_MLP_CACHE_PER_ROW;
-  // scratch: dA/dZ of the three hidden layers (reused) and weight-gradient partials
-  int64_t nch = (n + WG_ROWS - 1) / WG_ROWS;
-  float *d3, *d2, *d1, *part;
-  size_t act = (size_t)n * HID * sizeof(float);
-  size_t pbytes = (size_t)nch * (HID * HID + HID) * sizeof(float);
-  float* base;
-  if ((r = bp_ws(ctx, WS_MISC2, 3 * act + pbytes + 256, (void**)&base))) return r;
-  d3 = base;
-  d2 = d3 + (size_t)n * HID;
-  d1 = d2 + (size_t)n * HID;
-  part = d1 + (size_t)n * HID;
-  unsigned g = (unsigned)((n + ROWS - 1) / ROWS);
-  // layer 4: dW4, db4 from dy and A3; dZ3 = (dy W4) * GELU'(Z3)
-  k_wgrad<HID, OUT><<<(unsigned)nch, DT, 0, ctx->stream>>>(n, dy, OUT, cache + CA3, LC, part);
-  BP_LAUNCH_CHECK(ctx, "mlp wgrad 4");
-  k_sum_partials<<<(OUT * HID + OUT + 255) / 256, 256, 0, ctx->stream>>>(
-      part, nch, OUT * HID, OUT, grad + OFF_W4, grad + OFF_B4);
-  BP_LAUNCH_CHECK(ctx, "mlp sum 4");
-  k_dense<OUT, HID, true, 2><<<g, DT, 0, ctx->stream>>>(n, dy, OUT, params + OFF_W4, nullptr,
-                                                        cache + CZ3, LC, d3, HID, nullptr, 0);
-  BP_LAUNCH_CHECK(ctx, "mlp dgrad 3");
-  // layer 3
-  k_wgrad<HID, HID><<<(unsigned)nch, DT, 0, ctx->stream>>>(n, d3, HID, cache + CA2, LC, part);
-  BP_LAUNCH_CHECK(ctx, "mlp wgrad 3");
-  k_sum_partials<<<(HID * HID + HID + 255) / 256, 256, 0, ctx->stream>>>(
-      part, nch, HID * HID, HID, grad + OFF_W3, grad + OFF_B3);
-  BP_LAUNCH_CHECK(ctx, "mlp sum 3");
-  k_dense<HID, HID, true, 2><<<g, DT, 0, ctx->stream>>>(n, d3, HID, params + OFF_W3, nullptr,
-                                                        cache + CZ2, LC, d2, HID, nullptr, 0);
-  BP_LAUNCH_CHECK(ctx, "mlp dgrad 2");
-  // layer 2
-  k_wgrad<HID, HID><<<(unsigned)nch, DT, 0, ctx->stream>>>(n, d2, HID, cache + CA1, LC, part);
-  BP_LAUNCH_CHECK(ctx, "mlp wgrad 2");
-  k_sum_partials<<<(HID * HID + HID + 255) / 256, 256, 0, ctx->stream>>>(
-      part, nch, HID * HID, HID, grad + OFF_W2, grad + OFF_B2);
-  BP_LAUNCH_CHECK(ctx, "mlp sum 2");
-  k_dense<HID, HID, true, 2><<<g, DT, 0, ctx->stream>>>(n, d2, HID, params + OFF_W2, nullptr,
-                                                        cache + CZ1, LC, d1, HID, nullptr, 0);
-  BP_LAUNCH_CHECK(ctx, "mlp dgrad 1");
-  // layer 1
-  k_wgrad<IN, HID><<<(unsigned)nch, DT, 0, ctx->stream>>>(n, d1, HID, x, IN, part);
-  BP_LAUNCH_CHECK(ctx, "mlp wgrad 1");
-  k_sum_partials<<<(HID * IN + HID + 255) / 256, 256, 0, ctx->stream>>>(
-      part, nch, HID * IN, HID, grad + OFF_W1, grad + OFF_B1);
-  BP_LAUNCH_CHECK(ctx, "mlp sum 1");
+  const unsigned grid = mt_grid(ctx, n);
+  float* part;  // weight-gradient partials, one set per CTA
+  if ((r = bp_ws(ctx, WS_MISC2, (size_t)grid * NPAR * sizeof(float), (void**)&part))) return r;
+  BP_CUDA(ctx, cudaFuncSetAttribute(k_backward, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                    (int)sizeof(MtBackward)));
+  k_backward<<<grid, MT_THREADS, sizeof(MtBackward), ctx->stream>>>(n, x, params, cache, dy, part);
+  BP_LAUNCH_CHECK(ctx, "mlp backward");
+  k_sum_partials<<<(NPAR + SP_COLS - 1) / SP_COLS, SP_THREADS, 0, ctx->stream>>>(part, (int)grid,
+                                                                               grad);
+  BP_LAUNCH_CHECK(ctx, "mlp gradient sums");
   return BP_OK;
 }
 
