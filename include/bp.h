@@ -501,8 +501,8 @@ int bp_paste_halos_healpix(bp_ctx* ctx, int64_t n, const double* theta, const do
  * edges[b] <= |l| < edges[b + 1] (0 for an empty bin), nmodes[b] their count.  edges: HOST
  * FP64 [nb + 1], increasing from >= 0, nb in [1, 256] (the paper uses 30 logarithmic bins
  * over 1e2 < l < 1e5); cl: device FP64 [nb]; nmodes: device int64 [nb] or NULL.  FP64
- * throughout; deterministic.  Synchronises once (uploads twiddles and edges).  Errors:
- * BP_EINVAL (sizes, dtheta, edges, null pointer). */
+ * throughout; deterministic.  A context's first call uploads a table and synchronises; later
+ * calls do not.  Errors: BP_EINVAL (sizes, dtheta, edges, null pointer). */
 int bp_power_spectrum(bp_ctx* ctx, const float* map, const float* lo, int nx, int ny,
                       double dtheta, int nb, const double* edges, double* cl, int64_t* nmodes);
 

@@ -271,6 +271,7 @@ int bp_destroy(bp_ctx* ctx) {
     for (int q = 0; q < 2; ++q)
       if (ctx->ev[p][q]) cudaEventDestroy(ctx->ev[p][q]);
   if (ctx->table_mem) cudaFree(ctx->table_mem);
+  if (ctx->fft_tw) cudaFree(ctx->fft_tw);
   if (ctx->d_counter) cudaFree(ctx->d_counter);
   if (ctx->d_flags) cudaFree(ctx->d_flags);
   if (ctx->h_pinned) cudaFreeHost(ctx->h_pinned);

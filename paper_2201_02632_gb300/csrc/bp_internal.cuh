@@ -87,6 +87,7 @@ struct bp_ctx {
   BpTables t;
   cudaStream_t stream;
   void* table_mem;
+  void* fft_tw;  // twiddle table of the power spectrum (uploaded on its first use)
   void* ws[WS_NSLOTS];
   size_t ws_bytes[WS_NSLOTS];
   uint64_t ws_gen[WS_NSLOTS];  // calls of bp_ws per slot (every user of a slot asks for it)
