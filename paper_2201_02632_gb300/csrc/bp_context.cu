@@ -223,6 +223,7 @@ int bp_create(bp_ctx** out, const bp_cosmology* cosmo, const bp_icm_params* icm,
   P.alpha_nt = q.alpha_nt;
   P.beta_nt = q.beta_nt;
   P.n_nt = q.n_nt;
+  P.f_max = pow(4.0, -q.n_nt) / q.alpha_nt;
   P.energy_sign = q.energy_sign;
   P.field_fb = q.field_fb;
   P.CP = bpc::SIGMA_T / bpc::ME_C2_J * bpc::MSUN_KG * 1.0e6 / (bpc::MPC_M * bpc::MPC_M);

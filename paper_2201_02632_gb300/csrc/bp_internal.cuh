@@ -55,6 +55,7 @@ struct BpParams {
   double rho_cr0;            // Msun/Mpc^3
   // ICM
   double Gamma, n_poly, eps_dm, eps_star, f_star, S_star, alpha_nt, beta_nt, n_nt;
+  double f_max;  // 4^-n_nt / alpha_nt
   int energy_sign, field_fb;
   // observables: y per (P x length) and sigma_T n_e per (rho_g x length)
   double CP, CN;
