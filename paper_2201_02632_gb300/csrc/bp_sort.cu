@@ -42,19 +42,70 @@ __device__ T block_excl_scan(T v, T* total) {
   return res;
 }
 
+// A thread's SCAN_PER_THREAD counts from base on (zeros past n), 16 bytes at a time where in
+// allows it (a scan of part of an array may start anywhere).
+__device__ __forceinline__ int64_t scan_load(const uint32_t* __restrict__ in, int64_t base,
+                                             int64_t n, uint32_t (&v)[SCAN_PER_THREAD]) {
+  static_assert(SCAN_PER_THREAD == 8, "two 16-byte loads");
+  if (base + SCAN_PER_THREAD <= n && ((uintptr_t)in & 15) == 0) {
+    const uint4 a = *reinterpret_cast<const uint4*>(in + base);
+    const uint4 b = *reinterpret_cast<const uint4*>(in + base + 4);
+    v[0] = a.x, v[1] = a.y, v[2] = a.z, v[3] = a.w;
+    v[4] = b.x, v[5] = b.y, v[6] = b.z, v[7] = b.w;
+  } else {
+#pragma unroll
+    for (int k = 0; k < SCAN_PER_THREAD; ++k) v[k] = base + k < n ? in[base + k] : 0u;
+  }
+  int64_t s = 0;
+#pragma unroll
+  for (int k = 0; k < SCAN_PER_THREAD; ++k) s += v[k];
+  return s;
+}
+
+__device__ __forceinline__ void scan_store(int64_t* __restrict__ out, int64_t base, int64_t n,
+                                           const uint32_t (&v)[SCAN_PER_THREAD], int64_t ex) {
+  if (base + SCAN_PER_THREAD <= n && ((uintptr_t)out & 15) == 0) {
+#pragma unroll
+    for (int k = 0; k < SCAN_PER_THREAD; k += 2) {
+      const longlong2 w = make_longlong2(ex, ex + v[k]);
+      *reinterpret_cast<longlong2*>(out + base + k) = w;
+      ex += (int64_t)v[k] + v[k + 1];
+    }
+  } else {
+#pragma unroll
+    for (int k = 0; k < SCAN_PER_THREAD; ++k) {
+      if (base + k < n) out[base + k] = ex;
+      ex += v[k];
+    }
+  }
+}
+
+// A scan of a few chunks in one block, total included.
+__global__ void __launch_bounds__(SCAN_THREADS) k_scan_few(const uint32_t* in, int64_t n,
+                                                           int64_t* out) {
+  int64_t carry = 0;
+  for (int64_t c = 0; c < n; c += SCAN_CHUNK) {
+    const int64_t base = c + (int64_t)threadIdx.x * SCAN_PER_THREAD;
+    uint32_t v[SCAN_PER_THREAD];
+    int64_t tot;
+    const int64_t s = scan_load(in, base, n, v);
+    const int64_t ex = block_excl_scan<int64_t>(s, &tot) + carry;
+    scan_store(out, base, n, v, ex);
+    carry += tot;
+  }
+  if (threadIdx.x == 0) out[n] = carry;
+}
+
 __global__ void __launch_bounds__(SCAN_THREADS) k_scan_reduce(const uint32_t* in, int64_t n,
                                                               int64_t* bsum) {
-  int64_t base = (int64_t)blockIdx.x * SCAN_CHUNK + (int64_t)threadIdx.x * SCAN_PER_THREAD;
-  int64_t s = 0;
-  for (int k = 0; k < SCAN_PER_THREAD; ++k)
-    if (base + k < n) s += in[base + k];
+  const int64_t base = (int64_t)blockIdx.x * SCAN_CHUNK + (int64_t)threadIdx.x * SCAN_PER_THREAD;
+  uint32_t v[SCAN_PER_THREAD];
   int64_t tot;
-  block_excl_scan<int64_t>(s, &tot);
+  block_excl_scan<int64_t>(scan_load(in, base, n, v), &tot);
   if (threadIdx.x == 0) bsum[blockIdx.x] = tot;
 }
 
-// single block: in-place exclusive scan of nb block sums; writes the grand total
-// to bsum[nb]
+// single block: in-place exclusive scan of nb block sums
 __global__ void __launch_bounds__(SCAN_THREADS) k_scan_bsums(int64_t* bsum, int64_t nb) {
   __shared__ int64_t carry;
   if (threadIdx.x == 0) carry = 0;
@@ -69,24 +120,36 @@ __global__ void __launch_bounds__(SCAN_THREADS) k_scan_bsums(int64_t* bsum, int6
     if (threadIdx.x == 0) carry += tot;
     __syncthreads();
   }
-  if (threadIdx.x == 0) bsum[nb] = carry;
 }
 
+// summed: bsum holds the blocks' sums, not yet scanned: every block adds up the ones before it
 __global__ void __launch_bounds__(SCAN_THREADS) k_scan_down(const uint32_t* in, int64_t n,
-                                                            const int64_t* bsum, int64_t* out) {
-  int64_t base = (int64_t)blockIdx.x * SCAN_CHUNK + (int64_t)threadIdx.x * SCAN_PER_THREAD;
+                                                            const int64_t* bsum, bool summed,
+                                                            int64_t* out) {
+  const int64_t base = (int64_t)blockIdx.x * SCAN_CHUNK + (int64_t)threadIdx.x * SCAN_PER_THREAD;
   uint32_t v[SCAN_PER_THREAD];
-  int64_t s = 0;
-  for (int k = 0; k < SCAN_PER_THREAD; ++k) {
-    v[k] = (base + k < n) ? in[base + k] : 0u;
-    s += v[k];
+  const int64_t s = scan_load(in, base, n, v);
+  int64_t before;
+  if (summed) {
+    int64_t q = 0;
+    for (int64_t i = threadIdx.x; i < blockIdx.x; i += SCAN_THREADS) q += bsum[i];
+    block_excl_scan<int64_t>(q, &before);
+  } else {
+    before = bsum[blockIdx.x];
   }
-  int64_t ex = block_excl_scan<int64_t>(s, nullptr) + bsum[blockIdx.x];
-  for (int k = 0; k < SCAN_PER_THREAD; ++k) {
-    if (base + k < n) out[base + k] = ex;
-    ex += v[k];
-  }
+  int64_t tot;
+  const int64_t ex = block_excl_scan<int64_t>(s, &tot) + before;
+  scan_store(out, base, n, v, ex);
+  if (blockIdx.x == gridDim.x - 1 && threadIdx.x == 0) out[n] = before + tot;
 }
+
+// The scan's launches: what bounds a short one is their number.  Up to SCAN_FEW counts one block
+// does it (a chunk takes 2 us, a launch as much); up to SCAN_BLOCKS chunks every block adds up the
+// sums before it (at most 4 loads a thread); beyond, a block scans the sums first.  (With three
+// launches and a copy of the total for every scan, the deposit of 2e4 records took 43 launches
+// and copies, 253 us, now 217; pasting 1000 halos 48, 350 us, now 295.)
+constexpr int64_t SCAN_FEW = 2 * SCAN_CHUNK;
+constexpr int64_t SCAN_BLOCKS = 4 * SCAN_THREADS;
 
 // ---------------------------------------------------------------- radix sort
 constexpr int RS_THREADS = 256;
@@ -247,21 +310,10 @@ void rs_prefer_shared() {
 
 // exclusive scan of n u32 counts into out[0..n-1]; out[n] receives the total.
 int bp_scan_u32_to_i64(bp_ctx* ctx, const uint32_t* in, int64_t* out, int64_t n) {
-  int64_t nb = (n + SCAN_CHUNK - 1) / SCAN_CHUNK;
-  if (nb == 0) nb = 1;
   int64_t* bsum;
-  int r = bp_ws(ctx, WS_MISC, (size_t)(nb + 1) * sizeof(int64_t), (void**)&bsum);
+  int r = bp_ws(ctx, WS_MISC, (size_t)(n / SCAN_CHUNK + 2) * sizeof(int64_t), (void**)&bsum);
   if (r) return r;
-  k_scan_reduce<<<(unsigned)nb, SCAN_THREADS, 0, ctx->stream>>>(in, n, bsum);
-  BP_LAUNCH_CHECK(ctx, "scan reduce");
-  k_scan_bsums<<<1, SCAN_THREADS, 0, ctx->stream>>>(bsum, nb);
-  BP_LAUNCH_CHECK(ctx, "scan block sums");
-  k_scan_down<<<(unsigned)nb, SCAN_THREADS, 0, ctx->stream>>>(in, n, bsum, out);
-  BP_LAUNCH_CHECK(ctx, "scan down");
-  // total
-  BP_CUDA(ctx, cudaMemcpyAsync(out + n, bsum + nb, sizeof(int64_t), cudaMemcpyDeviceToDevice,
-                               ctx->stream));
-  return BP_OK;
+  return bp_scan_u32_to_i64_buf(ctx, in, out, n, bsum);
 }
 
 int bp_radix_sort_pairs(bp_ctx* ctx, uint32_t* keys, uint32_t* vals, uint32_t* keys_tmp,
@@ -319,16 +371,21 @@ int bp_tile_ranges(bp_ctx* ctx, const uint32_t* keys, int64_t n, int64_t n_tiles
 // bsum: >= (n / 8192 + 2) int64.
 int bp_scan_u32_to_i64_buf(bp_ctx* ctx, const uint32_t* in, int64_t* out, int64_t n,
                            int64_t* bsum) {
-  int64_t nb = (n + SCAN_CHUNK - 1) / SCAN_CHUNK;
-  if (nb == 0) nb = 1;
+  if (n <= SCAN_FEW) {
+    k_scan_few<<<1, SCAN_THREADS, 0, ctx->stream>>>(in, n, out);
+    BP_LAUNCH_CHECK(ctx, "scan");
+    return BP_OK;
+  }
+  const int64_t nb = (n + SCAN_CHUNK - 1) / SCAN_CHUNK;
+  const bool summed = nb <= SCAN_BLOCKS;
   k_scan_reduce<<<(unsigned)nb, SCAN_THREADS, 0, ctx->stream>>>(in, n, bsum);
   BP_LAUNCH_CHECK(ctx, "scan reduce");
-  k_scan_bsums<<<1, SCAN_THREADS, 0, ctx->stream>>>(bsum, nb);
-  BP_LAUNCH_CHECK(ctx, "scan block sums");
-  k_scan_down<<<(unsigned)nb, SCAN_THREADS, 0, ctx->stream>>>(in, n, bsum, out);
+  if (!summed) {
+    k_scan_bsums<<<1, SCAN_THREADS, 0, ctx->stream>>>(bsum, nb);
+    BP_LAUNCH_CHECK(ctx, "scan block sums");
+  }
+  k_scan_down<<<(unsigned)nb, SCAN_THREADS, 0, ctx->stream>>>(in, n, bsum, summed, out);
   BP_LAUNCH_CHECK(ctx, "scan down");
-  BP_CUDA(ctx, cudaMemcpyAsync(out + n, bsum + nb, sizeof(int64_t), cudaMemcpyDeviceToDevice,
-                               ctx->stream));
   return BP_OK;
 }
 
@@ -372,6 +429,7 @@ int bp_radix_sort_pairs_buf(bp_ctx* ctx, uint32_t* keys, uint32_t* vals, uint32_
 // first launch would otherwise load its code into device memory).
 int bp_sort_preload(bp_ctx* ctx) {
   cudaFuncAttributes a;
+  BP_CUDA(ctx, cudaFuncGetAttributes(&a, k_scan_few));
   BP_CUDA(ctx, cudaFuncGetAttributes(&a, k_scan_reduce));
   BP_CUDA(ctx, cudaFuncGetAttributes(&a, k_scan_bsums));
   BP_CUDA(ctx, cudaFuncGetAttributes(&a, k_scan_down));
