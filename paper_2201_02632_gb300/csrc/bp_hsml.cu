@@ -18,8 +18,8 @@
 //                  k_curve_final the particle ids and float4 positions into the last
 //  k_tree          boxes of one level from the positions, or from the level below
 //  k_hs_start      first search radius of every particle, a thread each
-//  k_hsml_group    one warp per 16 particles: one search for all of them, its particles in
-//                  shared memory; four particles' lists at a time solve N_eff(h) = N_ngb
+//  k_hsml_group    one warp per 8 particles: one search of the tree for all of them; four
+//                  particles' lists at a time solve N_eff(h) = N_ngb
 //  k_hsml          one warp per particle: the few that the groups leave, and large N_ngb; the
 //                  particles within R compacted into shared memory by ballot; R grows until
 //                  N_eff(R) >= N_ngb, then N_eff(h) = N_ngb is solved in (0, R] by Newton
@@ -27,7 +27,7 @@
 // Every list is in tree order and every sum lane-strided plus a fixed shuffle tree:
 // deterministic.
 //
-// What bounds it: instruction issue (57 % of the slots in k_hsml_group, the rest is waiting for
+// What bounds it: instruction issue (60 % of the slots in k_hsml_group, the rest is waiting for
 // leaves from L2).  4e6 light-cone particles, N_ngb = 64: 15.0 ms in all (30.4 ms with a warp per
 // particle that tests the Z-curve cells around it, found by binary searches: 6100 instructions
 // per particle, 1400 particles tested).

@@ -959,7 +959,7 @@ struct ThreadGas {
 // halo) every lane repeated it.  One thread per halo does it once, and the node tables leave 8
 // logarithms per halo.  Halos without a starting point are left to k_solve's nested iteration
 // (okv_nested).  Measured: 1e6 halos 4.1 ms (20.2 ms with eight lanes per halo; the FP64 pipe is
-// 86% busy), 2e5 halos 1.1 ms (4.9 ms).
+// 86% busy), 2e5 halos 1.1 ms (5.7 ms).
 __global__ void __launch_bounds__(128) k_polish(
     BpParams P, int64_t n, double* model, int32_t* status, double tol, int64_t* nbad,
     int64_t* nfallback, SolveExtra X, const Halo* __restrict__ halos,
