@@ -336,18 +336,23 @@ __device__ __forceinline__ void neff_quarter(float* l, int len, int steps, float
 }
 
 // one Newton step on ln N_eff(ln h) = ln n_ngb (nearly linear) from x inside the bisection
-// bracket [lo, hi]; h: the answer so far; false: it is the last
+// bracket [lo, hi]; h: the answer so far; step: the last step's length (infinite at first);
+// false: it is the last.  A step that is not half as long as the last is a bisection: with a clump
+// between x and the root, Newton can jump to and fro between its two sides, both within the
+// bracket, for ever (light-cone particles, N_ngb = 200: 3 in 1e5).
 __device__ __forceinline__ bool newton(float n_ngb, float f, float df, float& x, float& lo,
-                                       float& hi, float& h) {
+                                       float& hi, float& h, float& step) {
   const float F = f - n_ngb;
   if (F < 0.f) lo = x; else hi = x;
   h = x;
   if (fabsf(F) <= 1e-6f * n_ngb) return false;
   float xn = (df > 0.f) ? x * __expf(__logf(n_ngb / f) * f / (x * df)) : 0.f;
-  const bool in = xn > lo && xn < hi;
+  const bool in = xn > lo && xn < hi && fabsf(xn - x) < 0.5f * step;
   if (!in) xn = 0.5f * (lo + hi);
-  // (a Newton step leaves about its square)
-  const bool last = fabsf(xn - x) <= (in ? 2e-4f : 1e-6f) * x || hi - lo <= 1e-6f * hi;
+  step = fabsf(xn - x);
+  // what a Newton step leaves is of the order of its square; next to it the FP32 sums' rounding
+  // is the larger part (stopping at 1e-6 instead leaves the same errors, at 0.6 more steps)
+  const bool last = step <= (in ? 2e-4f : 1e-6f) * x || hi - lo <= 1e-6f * hi;
   h = x = xn;
   return !last;
 }
@@ -581,12 +586,12 @@ __global__ void __launch_bounds__(32)
         __syncwarp();
         const bool found = has && f >= n_ngb;
         bool run = found && f - n_ngb >= 1e-6f * n_ngb;
-        float h = Rq, xlo = 0.f, xhi = Rq;
+        float h = Rq, xlo = 0.f, xhi = Rq, step = INFINITY;
         float x = run ? fminf(Rq, fmaxf(0.5f * Rq, Rq * cbrtf(n_ngb / f))) : Rq;
         const float f_R = f;
         for (int it = 0; it < 40 && __any_sync(ALL, run); ++it) {
           neff_quarter<false>(l, len, steps, x, sub, f, df);
-          if (run) run = newton(n_ngb, f, df, x, xlo, xhi, h);
+          if (run) run = newton(n_ngb, f, df, x, xlo, xhi, h, step);
         }
         // back to the particles' lanes
         bool gone = false;
@@ -705,11 +710,12 @@ __global__ void __launch_bounds__(32)
     // N_eff(R) >= n_ngb: the root in (0, R]
     h = R;
     if (f - n_ngb >= 1e-6f * n_ngb) {
-      float lo = 0.f, hi = R, x = fminf(R, fmaxf(0.5f * R, R * cbrtf(n_ngb / f)));
+      float lo = 0.f, hi = R, step = INFINITY;
+      float x = fminf(R, fmaxf(0.5f * R, R * cbrtf(n_ngb / f)));
       for (int it = 0; it < 40; ++it) {
         if (stream) neff_stream(tree, pos, p, R, x, lane, f, df);
         else neff<false>(buf, total, x, lane, f, df);
-        if (!newton(n_ngb, f, df, x, lo, hi, h)) break;
+        if (!newton(n_ngb, f, df, x, lo, hi, h, step)) break;
       }
     }
     done = true;

@@ -1,0 +1,42 @@
+"""Smoothing lengths from search radii that the solve has trouble with.
+
+Tolerance: that of the other smoothing-length tests, 1e-5 (FP32 sums of at most 4096 positive
+weights, relative error below 4e-6; N_eff grows like h^3 or faster)."""
+import numpy as np
+import pytest
+import torch
+
+from tests.gpu_common import api, ctx, cuda  # noqa: F401
+
+pytestmark = pytest.mark.gpu
+RTOL = 1e-5
+
+
+def _gpu(ctx, p, n_ngb, guess=None):
+    h = ctx.smoothing_lengths(cuda(p[0]), cuda(p[1]), cuda(p[2]), n_ngb,
+                              guess=None if guess is None else cuda(guess, torch.float32))
+    return h.double().cpu().numpy()
+
+
+def _beside_a_clump(seed):
+    """Particle 0 in a uniform field with one dense clump near the edge of its kernel."""
+    rng = np.random.default_rng(seed)
+    m = int(40 * np.exp(rng.uniform(0, 4)))
+    d = rng.uniform(3, 8)
+    s = d * 10 ** rng.uniform(-3, -0.7)
+    field = rng.uniform(-10, 10, (3, 1500))
+    field[:, 0] = 0
+    dr = rng.normal(size=3)
+    dr /= np.linalg.norm(dr)
+    return np.concatenate([field, d * dr[:, None] + rng.normal(0, s, (3, m))], 1).astype(np.float32)
+
+
+# the first radius is 1.25 x the guess; from 1.5 h, Newton's steps jump over the clump and back
+@pytest.mark.parametrize("seed", [17, 912, 1262, 2493])
+@pytest.mark.parametrize("first", [1.3, 1.5, 2.0])
+def test_newton_steps_over_a_clump_and_back(orc, api, ctx, seed, first):
+    p = _beside_a_clump(seed)
+    h = orc.smoothing_lengths_at(*p, np.arange(1), 200.0)
+    guess = np.full(p.shape[1], np.nan)
+    guess[0] = first * h[0] / 1.25
+    np.testing.assert_allclose(_gpu(ctx, p, 200.0, guess)[:1], h, rtol=RTOL)
