@@ -49,6 +49,7 @@ constexpr int HS_CAP = 2048;          // candidate distances per warp (shared me
 constexpr int HS_MAX_ROUNDS = 48;     // radius updates per particle
 constexpr int HS_QBITS = 21;          // quantisation bits per axis (63-bit keys)
 constexpr int HS_SCAN_CAPS = 16;      // particles worth one search, in buffer capacities
+constexpr float HS_FAR = 1.5f;        // a guess is looked at above this many leaf diagonals
 // The groups.  A search shared by 8 or 16 particles costs the same (13.6 ms at 4e6 particles,
 // 32: 15 ms; at 5e4, 8 leaves more warps: 0.22 and 0.33 ms).  Lists of 2 N_ngb to 3 N_ngb: 13.6
 // ms, 4 N_ngb 15.5 ms (fewer warps per SM).  Starts of 0.3 N_ngb to 0.5 N_ngb particles: 13.6 to
@@ -358,7 +359,12 @@ __device__ __forceinline__ bool newton(float n_ngb, float f, float df, float& x,
 }
 
 // First radius of every particle (curve order), a thread each: 1.25 x the caller's guess, or
-// from the distances to the particles around it on the curve (spatial neighbours, mostly).
+// from the distances to the particles around it on the curve (spatial neighbours, mostly).  A
+// guess far above the size of the particle's leaf (32 particles), and above four times what those
+// distances give, would only be searched in vain, thousands of particles a time: it is left.
+// (1e5 particles, N_ngb = 64, with and without this: guesses of h 0.68 and 0.67 ms, of 10 h 1.3 and
+// 8.1 ms, of 1000 h 1.2 and 129 ms.)  Not with so few particles that h can be any multiple of
+// their extent.
 __global__ void __launch_bounds__(128)
     k_hs_start(int64_t n, const float4* __restrict__ pos, const uint32_t* __restrict__ ids, Cube cb,
                float n_ngb, const float* __restrict__ guess, float* R0) {
@@ -375,7 +381,16 @@ __global__ void __launch_bounds__(128)
     const float gv = guess[ids[kk]];
     if (gv > 0.f && isfinite(gv)) R = 1.25f * gv;
   }
-  if (__any_sync(ALL, R == 0.f)) {
+  float far = INFINITY;
+  if (guess && n_ngb < (float)n) {
+    const auto extent = [&](float v) {
+      const unsigned o = ordered(v);
+      return unordered(__reduce_max_sync(ALL, o)) - unordered(__reduce_min_sync(ALL, o));
+    };
+    const float4 e = make_float4(extent(p.x), extent(p.y), extent(p.z), 0.f);
+    far = HS_FAR * sqrtf(dist2(e, make_float4(0.f, 0.f, 0.f, 0.f))) * cbrtf(n_ngb / 64.0f);
+  }
+  if (__any_sync(ALL, R == 0.f || R > far)) {
     // the median distance to the 64 particles around the warp's on the curve, scaled to
     // hold HG_START N_ngb particles at that density
     const int W = n < 64 ? (int)n : 64;
@@ -402,8 +417,9 @@ __global__ void __launch_bounds__(128)
       for (int j = 0; j < W; ++j) cnt += list[j * 32] <= cf;
       if (2 * cnt > W) b = c; else a = c;
     }
-    if (R == 0.f)
-      R = fmaxf(sqrtf(__uint_as_float(b)) * cbrtf(2.0f * HG_START * n_ngb / (float)W), cb.s);
+    const float E =
+        fmaxf(sqrtf(__uint_as_float(b)) * cbrtf(2.0f * HG_START * n_ngb / (float)W), cb.s);
+    if (R == 0.f || (R > far && R > 4.0f * E)) R = E;
   }
   if (k < n) R0[k] = R;
 }
@@ -650,6 +666,7 @@ __global__ void __launch_bounds__(32)
   const uint32_t id = ids[k];
   float R = left_k ? left_R[item] : R0[k];
   float r_short = 0.f, r_over = INFINITY;  // N_eff too small at r_short; too many at r_over
+  float cut = 0.63f;  // next cut of a radius with far too many particles
   float h = __int_as_float(0x7fc00000);
   bool done = false;
   for (int round = 0; round < HS_MAX_ROUNDS && !done; ++round) {
@@ -678,8 +695,9 @@ __global__ void __launch_bounds__(32)
     });
     __syncwarp();
     if (off > (uint32_t)(HS_SCAN_CAPS * cap)) {  // far too many: try a smaller radius first
-      const float Rn = 0.63f * R;
-      if (Rn > r_short) {
+      const float Rn = (r_short > 0.f ? 0.63f : cut) * R;
+      if (Rn > r_short) {  // (how many is not known: the cuts get deeper until one is too deep)
+        cut = fmaxf(cut * cut, 0.02f);
         R = Rn;
         __syncwarp();
         continue;

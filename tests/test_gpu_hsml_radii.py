@@ -6,6 +6,7 @@ import numpy as np
 import pytest
 import torch
 
+from paper_2201_02632_gb300 import inputs as I
 from tests.gpu_common import api, ctx, cuda  # noqa: F401
 
 pytestmark = pytest.mark.gpu
@@ -40,3 +41,41 @@ def test_newton_steps_over_a_clump_and_back(orc, api, ctx, seed, first):
     guess = np.full(p.shape[1], np.nan)
     guess[0] = first * h[0] / 1.25
     np.testing.assert_allclose(_gpu(ctx, p, 200.0, guess)[:1], h, rtol=RTOL)
+
+
+def _cone(n):
+    """Light-cone particles, more than one search of the one-warp kernel may meet (65536)."""
+    lc = I.lightcone(n_part=n, n_halo=n // 1333, side_deg=2.0, zr=(0.05, 1.5), seed=I.SEED_BASE + 78)
+    return np.stack([lc.parts["x"], lc.parts["y"], lc.parts["z"]])
+
+
+@pytest.mark.parametrize("n_ngb", [64.0, 200.0])
+def test_guesses_of_another_size(orc, api, ctx, n_ngb):
+    p = _cone(80000)
+    h = _gpu(ctx, p, n_ngb)
+    idx = np.random.default_rng(1).choice(h.size, 30, replace=False)
+    np.testing.assert_allclose(h[idx], orc.smoothing_lengths_at(*p, idx, n_ngb), rtol=RTOL)
+    for factor in (1e-6, 0.1, 4.0, 10.0, 1e3, 1e10, 1e30, 1e38):
+        guess = np.minimum(h * factor, 3e38)
+        np.testing.assert_allclose(_gpu(ctx, p, n_ngb, guess), h, rtol=2 * RTOL)
+
+
+def test_far_too_large_guesses_cost_little(api, ctx):
+    """A guess in other units (1000 h) takes about as long as none; 5 times that is allowed (it was
+    100 times: every search read tens of thousands of particles)."""
+    x = [cuda(v) for v in _cone(100000)]
+    h = ctx.smoothing_lengths(*x, 64.0)
+
+    def ms(guess):
+        best = float("inf")
+        for _ in range(5):
+            e0, e1 = (torch.cuda.Event(enable_timing=True) for _ in range(2))
+            e0.record()
+            ctx.smoothing_lengths(*x, 64.0, guess=guess)
+            e1.record()
+            torch.cuda.synchronize()
+            best = min(best, e0.elapsed_time(e1))
+        return best
+
+    none, far = ms(None), ms(1000.0 * h)
+    assert far <= 5.0 * none, (far, none)
