@@ -639,7 +639,8 @@ __global__ void __launch_bounds__(32)
   leave(act);
 }
 
-// One warp per particle: every particle of a call with a large N_ngb, or the ones that the groups
+// One warp per particle: every particle of a call with a large N_ngb (a block each, as far as the
+// grid goes), or the ones that the groups
 // left (5 % in a light-cone: field particles with a halo at the edge of their kernel, hundreds of
 // candidates of little weight), fetched one by one.
 __global__ void __launch_bounds__(32)
@@ -653,7 +654,7 @@ __global__ void __launch_bounds__(32)
   float* buf = s_dyn;
   // every particle, or the ones the groups left
   const int64_t todo = left_k ? (int64_t)*n_left : n;
-  for (int64_t item = blockIdx.x;;) {
+  for (int64_t item = blockIdx.x;; item += gridDim.x) {
     if (left_k) {  // (their work varies by orders of magnitude)
       unsigned long long q = 0;
       if (lane == 0) q = atomicAdd(next, 1ull);
@@ -744,7 +745,6 @@ __global__ void __launch_bounds__(32)
     if (!done) atomicAdd((unsigned long long*)nfail, 1ull);
   }
   __syncwarp();
-  if (!left_k) break;
   }
 }
 
@@ -870,9 +870,9 @@ extern "C" int bp_smoothing_lengths(bp_ctx* ctx, int64_t n, const float* x, cons
     BP_LAUNCH_CHECK(ctx, "smoothing lengths of groups");
     left_k = A;
     left_R = (const float*)B;
-    blocks = std::min(blocks, (int64_t)ctx->num_sms * 26);
+    blocks = std::min(blocks, (int64_t)ctx->num_sms * 26);  // (they fetch their particles)
   }
-  k_hsml<<<(unsigned)blocks, 32, smem, ctx->stream>>>(
+  k_hsml<<<bp_item_grid(blocks), 32, smem, ctx->stream>>>(
       n, pos, tree, E, (float)n_ngb, cap, (const float*)F, left_k, left_R, n_left, n_left + 1, h_out,
       ctx->d_counter + 5);
   BP_LAUNCH_CHECK(ctx, "smoothing lengths");

@@ -7,6 +7,8 @@
 #include <stdint.h>
 #include <stdio.h>
 
+#include <algorithm>
+
 #include "../../include/bp.h"
 
 // ---------------------------------------------------------------- constants
@@ -136,6 +138,10 @@ void bp_phase_end(bp_ctx* ctx, int ph);
 int bp_fail(bp_ctx* ctx, int code, const char* fmt, ...);
 int bp_cuda_check(bp_ctx* ctx, cudaError_t e, const char* what);
 int bp_ws(bp_ctx* ctx, int slot, size_t bytes, void** out);
+
+// Blocks of a launch with one block per item that strides over the rest: at most the largest
+// grid (2^31 - 1 blocks).
+inline unsigned bp_item_grid(int64_t n) { return (unsigned)std::min<int64_t>(n, 0x7fffffff); }
 
 // Threads per block of a one-thread-per-item launch: `big`, or one warp per block when
 // blocks of `big` would cover fewer SMs than the GPU has.  Scalar FP64 work is bound by each
