@@ -14,9 +14,9 @@
 // in the others.
 //
 // Kernels: k_setup (the scalar set-up, one thread per halo), k_start (the reduced problem in
-// FP32 to its rounding floor: starting points; one thread per halo), k_polish (FP64: a
-// two-dimensional Newton in (ln T, ln r_f) from the starting point, one quadrature per step, to
-// the tolerance; one thread per halo), k_solve (the nested iteration, a warp per halo, for halos
+// FP32 to its rounding floor: starting points; one thread per halo, eight in small catalogues),
+// k_polish (FP64: a two-dimensional Newton in (ln T, ln r_f) from the starting point, one
+// quadrature per step, to the tolerance; threads as k_start), k_solve (the nested iteration, a warp per halo, for halos
 // without a starting point), then k_setup + k_solve again, nested, for halos the Newton did not
 // bring in (the fallback).  BP_SOLVE_FP32_GATED: k_presolve or k_start, then k_accept32.
 #include <algorithm>
@@ -522,6 +522,11 @@ __device__ bool halo_setup(const BpParams& P, const BpTables& TB, int64_t n, int
 }
 
 constexpr int SOLVE_WARPS = 4;  // warps per block
+// Halos per SM up to which k_start and k_polish take eight threads a halo: one thread per halo is a
+// long serial chain that a small catalogue cannot hide, eight threads repeat the scalar part.  The
+// whole solve with eight threads and with one: 40 halos 195 and 266 us, 1000 halos 206 and 298,
+// 3000 halos 245 and 336, 6000 halos (39 per SM) 321 and 311, 2e4 halos 645 and 423 us.
+constexpr int SOLVE_FEW = 32;
 // |R_e| below which the nested iteration hands over to the two-dimensional Newton
 constexpr double NEWTON2D_SWITCH = 1e-3;
 
@@ -824,13 +829,15 @@ __global__ void __launch_bounds__(32 * SOLVE_WARPS) k_solve(
   }
 }
 
-// ---------------------------------------------------------------- one thread per halo
-// The gas integrals over [0, r_f] by one thread, in FP32 or FP64 (Real).  Region A's complete
-// panels come from the node tables, so only the panel that c (or r_f) cuts needs a logarithm per
-// node; region B ([r_vir, r_f], doubling panels) needs a reciprocal per node.  Only
+// ---------------------------------------------------------------- one thread per halo, or eight
+// The gas integrals over [0, r_f] by W threads (1 or 8), in FP32 or FP64 (Real).  Region A's
+// complete panels come from the node tables, so only the panel that c (or r_f) cuts needs a
+// logarithm per node; region B ([r_vir, r_f], doubling panels) needs a reciprocal per node.  Only
 //   I_k = int theta^k r^2 dr,  k = n - 1, n, n + 1,
 // is summed: Phi = Phi0 + (n + 1) T (1 - theta) turns the sums with Phi into differences of
-// these.  Sums run panel by panel (a panel's eight terms first).
+// these.  Sums run panel by panel (a panel's eight terms first).  With eight threads each takes a
+// panel and every one of them adds up the panels in the same order; products and sums are rounded
+// as written, so that both forms give the same bits.
 template <typename Real>
 struct Sums3 {
   Real m, n, p;  // k = n - 1, n, n + 1
@@ -839,6 +846,10 @@ __device__ __forceinline__ double t_log1p(double x) { return log1p(x); }
 __device__ __forceinline__ float t_log1p(float x) { return log1pf(x); }
 __device__ __forceinline__ double t_pow(double x, double y) { return pow(x, y); }
 __device__ __forceinline__ float t_pow(float x, float y) { return powf(x, y); }
+__device__ __forceinline__ double t_fma(double x, double y, double z) { return __fma_rn(x, y, z); }
+__device__ __forceinline__ float t_fma(float x, float y, float z) { return __fmaf_rn(x, y, z); }
+__device__ __forceinline__ double t_mul(double x, double y) { return __dmul_rn(x, y); }
+__device__ __forceinline__ float t_mul(float x, float y) { return __fmul_rn(x, y); }
 __device__ __forceinline__ double tab_g(double, int k) { return c_ag[k]; }
 __device__ __forceinline__ float tab_g(float, int k) { return c_agf[k]; }
 __device__ __forceinline__ double tab_w(double, int k) { return c_aw[k]; }
@@ -852,17 +863,17 @@ __device__ __forceinline__ float tab_w8(float, int j) { return c_glwf[j]; }
 template <typename Real>
 __device__ __forceinline__ Real theta_pow(Real th, Real n, int n_int, int k_off) {
   if (n_int == 5) {  // the default polytrope (Gamma = 1.2)
-    const Real t2 = th * th;
-    Real r = t2 * t2;
-    for (int k = 0; k < k_off; ++k) r *= th;
+    const Real t2 = t_mul(th, th);
+    Real r = t_mul(t2, t2);
+    for (int k = 0; k < k_off; ++k) r = t_mul(r, th);
     return r;
   }
   if (n_int > 0) {
     int e = n_int - 1 + k_off;
     Real r = 1, b = th;
     while (e) {
-      if (e & 1) r *= b;
-      b *= b;
+      if (e & 1) r = t_mul(r, b);
+      b = t_mul(b, b);
       e >>= 1;
     }
     return r;
@@ -870,26 +881,38 @@ __device__ __forceinline__ Real theta_pow(Real th, Real n, int n_int, int k_off)
   return t_pow(th, n - 1 + k_off);
 }
 
-template <typename Real>
+template <typename Real, int W>
 struct ThreadGas {
+  static_assert(W == 1 || W == NGT, "one thread, or one per node and per panel");
   Real c, rvir, rs, phi0, GM, psi;  // psi = G M / (m(c) r_s): Phi - Phi0 = psi g(x) inside r_vir
   Real n;
   int n_int;
   int nfull;         // complete panels of region A
   Real cg[NGT], cw[NGT];  // nodes of the panel that c cuts (weight 0: none)
 
+  // the W threads of a halo (aligned in the warp)
+  __device__ __forceinline__ static int at() { return threadIdx.x & (W - 1); }
+  __device__ __forceinline__ static unsigned group() {
+    return ((1u << W) - 1u) << (threadIdx.x & 31 & ~(W - 1));
+  }
   __device__ __forceinline__ void acc(Sums3<Real>& s, Real w, Real th) const {
-    Real t = w * theta_pow(th, n, n_int, 0);
-    s.m += t;
-    t *= th;
-    s.n += t;
-    t *= th;
-    s.p += t;
+    const Real t = theta_pow(th, n, n_int, 0);
+    const Real tm = t_mul(w, t), tn = t_mul(tm, th);
+    s.m = t_fma(w, t, s.m);
+    s.n = t_fma(tm, th, s.n);
+    s.p = t_fma(tn, th, s.p);
   }
   __device__ __forceinline__ static void add(Sums3<Real>& s, const Sums3<Real>& v, Real f) {
-    s.m += f * v.m;
-    s.n += f * v.n;
-    s.p += f * v.p;
+    s.m = t_fma(f, v.m, s.m);
+    s.n = t_fma(f, v.n, s.n);
+    s.p = t_fma(f, v.p, s.p);
+  }
+  // node j of the panel of half width hw around mid (in x): g and weight
+  __device__ __forceinline__ static void node(Real mid, Real hw, int j, Real& g, Real& w) {
+    const Real x = t_fma(hw, tab_x8(Real(), j), mid);
+    w = t_mul(t_mul(t_mul(hw, tab_w8(Real(), j)), x), x);
+    // ln(1 + x) / x -> 1 - x / 2 for a panel of negligible width at the centre
+    g = x < (Real)1e-6 ? (Real)0.5 * x : (Real)1 - t_log1p(x) / x;
   }
   // complete panels below xa, and the nodes of the panel xa cuts (in x)
   __device__ int cut(Real xa, Real (&g)[NGT], Real (&w)[NGT]) const {
@@ -901,16 +924,33 @@ struct ThreadGas {
       ++p;
     }
     const Real hw = p < MAX_PANEL_A ? (Real)0.5 * (xa - lo) : (Real)0, mid = lo + hw;
+    if constexpr (W == 1) {
 #pragma unroll
-    for (int j = 0; j < NGT; ++j) {
-      const Real x = mid + hw * tab_x8(Real(), j);
-      w[j] = hw * tab_w8(Real(), j) * x * x;
-      // ln(1 + x) / x -> 1 - x / 2 for a panel of negligible width at the centre
-      g[j] = x < (Real)1e-6 ? (Real)0.5 * x : (Real)1 - t_log1p(x) / x;
+      for (int j = 0; j < NGT; ++j) node(mid, hw, j, g[j], w[j]);
+    } else {
+      Real gj, wj;
+      node(mid, hw, at(), gj, wj);
+#pragma unroll
+      for (int j = 0; j < NGT; ++j) {
+        g[j] = __shfl_sync(group(), gj, j, W);
+        w[j] = __shfl_sync(group(), wj, j, W);
+      }
     }
     return p;
   }
   __device__ void init() { nfull = cut(c, cg, cw); }
+  // Panel p of region B (p < MAX_PANEL_B, its start below r_f): its sums, returns its half width
+  __device__ __forceinline__ Real panel_b(int p, Real rf, Real t0, Real t1, Sums3<Real>& v) const {
+    const Real a = rvir * (Real)(1 << p);
+    const Real b = (Real)2 * a < rf ? (Real)2 * a : rf;
+    const Real mid = (Real)0.5 * (a + b), hw = (Real)0.5 * (b - a);
+#pragma unroll
+    for (int j = 0; j < NGT; ++j) {
+      const Real r = t_fma(hw, tab_x8(Real(), j), mid);
+      acc(v, t_mul(t_mul(tab_w8(Real(), j), r), r), t0 + t1 / r);
+    }
+    return hw;
+  }
   // Integrals over [0, rf] with theta = 1 + (Phi0 - Phi) inv_n1T
   __device__ Sums3<Real> integrals(Real rf, Real inv_n1T) const {
     Sums3<Real> s = {0, 0, 0};
@@ -919,63 +959,89 @@ struct ThreadGas {
     const bool full = rf >= rvir;
     Real g2[NGT], w2[NGT];
     if (!full) np = cut(rf / rs, g2, w2);
-    for (int p = 0; p < np; ++p) {
-      Sums3<Real> v = {0, 0, 0};
-#pragma unroll
-      for (int j = 0; j < NGT; ++j)
-        acc(v, tab_w(Real(), p * NGT + j), (Real)1 - q * tab_g(Real(), p * NGT + j));
-      add(s, v, rs3);
-    }
-    {
-      Sums3<Real> v = {0, 0, 0};
-#pragma unroll
-      for (int j = 0; j < NGT; ++j)
-        acc(v, full ? cw[j] : w2[j], (Real)1 - q * (full ? cg[j] : g2[j]));
-      add(s, v, rs3);
-    }
-    if (full) {
-      const Real t0 = (Real)1 + phi0 * inv_n1T, t1 = GM * inv_n1T;  // theta = t0 + t1 / r
-      Real a = rvir;
-      for (int p = 0; p < MAX_PANEL_B && a < rf; ++p) {
-        const Real b = (Real)2 * a < rf ? (Real)2 * a : rf;
-        const Real mid = (Real)0.5 * (a + b), hw = (Real)0.5 * (b - a);
+    // theta = t0 + t1 / r in region B
+    const Real t0 = t_fma(phi0, inv_n1T, (Real)1), t1 = GM * inv_n1T;
+    if constexpr (W == 1) {
+      for (int p = 0; p < np; ++p) {
         Sums3<Real> v = {0, 0, 0};
 #pragma unroll
-        for (int j = 0; j < NGT; ++j) {
-          const Real r = mid + hw * tab_x8(Real(), j);
-          acc(v, tab_w8(Real(), j) * r * r, t0 + t1 / r);
+        for (int j = 0; j < NGT; ++j)
+          acc(v, tab_w(Real(), p * NGT + j), t_fma(-q, tab_g(Real(), p * NGT + j), (Real)1));
+        add(s, v, rs3);
+      }
+      {
+        Sums3<Real> v = {0, 0, 0};
+#pragma unroll
+        for (int j = 0; j < NGT; ++j)
+          acc(v, full ? cw[j] : w2[j], t_fma(-q, full ? cg[j] : g2[j], (Real)1));
+        add(s, v, rs3);
+      }
+      if (full) {
+        for (int p = 0; p < MAX_PANEL_B && rvir * (Real)(1 << p) < rf; ++p) {
+          Sums3<Real> v = {0, 0, 0};
+          const Real hw = panel_b(p, rf, t0, t1, v);
+          add(s, v, hw);
         }
-        add(s, v, hw);
-        a = b;
+      }
+    } else {
+      int nt = np + 1;  // panels: np + 1 of region A, then those of region B
+      if (full)
+        for (int p = 0; p < MAX_PANEL_B && rvir * (Real)(1 << p) < rf; ++p) ++nt;
+      for (int p0 = 0; p0 < nt; p0 += W) {
+        const int p = p0 + at();
+        Sums3<Real> v = {0, 0, 0};
+        Real f = rs3;
+        if (p <= np) {
+          const int k = (p < np ? p : 0) * NGT;
+#pragma unroll
+          for (int j = 0; j < NGT; ++j) {
+            const Real w = p < np ? tab_w(Real(), k + j) : full ? cw[j] : w2[j];
+            const Real g = p < np ? tab_g(Real(), k + j) : full ? cg[j] : g2[j];
+            acc(v, w, t_fma(-q, g, (Real)1));
+          }
+        } else if (p < nt) {
+          f = panel_b(p - np - 1, rf, t0, t1, v);
+        }
+        __syncwarp(group());
+        for (int k = 0; k < W && p0 + k < nt; ++k) {
+          Sums3<Real> u;
+          u.m = __shfl_sync(group(), v.m, k, W);
+          u.n = __shfl_sync(group(), v.n, k, W);
+          u.p = __shfl_sync(group(), v.p, k, W);
+          add(s, u, __shfl_sync(group(), f, k, W));
+        }
       }
     }
     return s;
   }
 };
 
-// The FP64 two-dimensional Newton of k_solve from a starting point, one thread per halo.  FP64
+// The FP64 two-dimensional Newton of k_solve from a starting point, W threads per halo.  FP64
 // instructions cost this GPU 16 SM cycles per warp, whatever the active lanes, and most of an
 // evaluation is per-halo scalar work: with lanes over the quadrature nodes (eight lanes per
-// halo) every lane repeated it.  One thread per halo does it once, and the node tables leave 8
-// logarithms per halo.  Halos without a starting point are left to k_solve's nested iteration
-// (okv_nested).  Measured: 1e6 halos 4.1 ms (20.2 ms with eight lanes per halo; the FP64 pipe is
-// 86% busy), 2e5 halos 1.1 ms (5.7 ms).
+// halo) every lane repeats it.  One thread per halo does it once, and the node tables leave 8
+// logarithms per halo; eight threads share the panels of a catalogue too small to fill the GPU
+// (SOLVE_FEW).  Halos without a starting point are left to k_solve's nested iteration
+// (okv_nested).  Measured with one thread: 1e6 halos 4.1 ms (20.2 ms with eight lanes per halo
+// over the nodes; the FP64 pipe is 86% busy), 2e5 halos 1.1 ms (5.7 ms).
+template <int W>
 __global__ void __launch_bounds__(128) k_polish(
     BpParams P, int64_t n, double* model, int32_t* status, double tol, int64_t* nbad,
     int64_t* nfallback, SolveExtra X, const Halo* __restrict__ halos,
     const int32_t* __restrict__ okv, int32_t* okv_nested) {
-  const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= n || !okv[i]) return;
+  const int64_t i = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) / W;
+  if (i >= n || !okv[i]) return;  // (all threads of a halo together)
   const double g0 = X.guess[i], g1 = X.guess[n + i];
   const double eg1 = exp(g1);
+  const bool first = threadIdx.x % W == 0;  // the thread that writes
   if (!(isfinite(g0) && isfinite(g1) && eg1 > 0.0)) {
-    okv_nested[i] = 1;
+    if (first) okv_nested[i] = 1;
     return;
   }
   const Halo h = halos[i];
   const double nn = P.n_poly;
   const double rn_ = rint(nn);
-  ThreadGas<double> S;
+  ThreadGas<double, W> S;
   S.c = h.c;
   S.rvir = h.rvir;
   S.rs = h.rs;
@@ -1069,6 +1135,7 @@ __global__ void __launch_bounds__(128) k_polish(
     st = pass ? BP_HALO_OK : BP_HALO_FALLBACK;
   }
   if (eok && ethf <= 0.0) st = BP_HALO_THETA;
+  if (!first) return;
   auto put = [&](int f, double v) { model[(int64_t)f * n + i] = v; };
   put(BP_M_T, eok ? eT : 0.0);
   put(BP_M_RHO0, eok ? erho0 : 0.0);
@@ -1385,17 +1452,18 @@ __global__ void __launch_bounds__(32 * SOLVE_WARPS) k_presolve(
 }
 
 // The pre-solve of every mode but the gated one without a seed: the same iteration as k_presolve,
-// one thread per halo with the tabulated nodes (no shuffles, no scalar work repeated in 32
+// W threads per halo (as k_polish) with the tabulated nodes (no shuffles, no scalar work repeated in 32
 // lanes, no logarithm per node).  A warp runs as long as its slowest halo.  Measured from the
 // default start: 1e6 halos 1.4 ms (k_presolve: 11.2 ms).  It sums in another order than
 // k_presolve, which moves the FP32 solutions within their rounding floor (1e-6 relative); the
 // gated mode without a seed returns those solutions as its answer and keeps k_presolve, so that
 // its results stay what they are.
+template <int W>
 __global__ void __launch_bounds__(128) k_start(BpParams P, int64_t n, SolveExtra X,
                                                const Halo* __restrict__ halos,
                                                const int32_t* __restrict__ okv, double* guess,
                                                float* res32) {
-  const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  const int64_t i = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) / W;
   if (i >= n) return;
   float g0 = __int_as_float(0x7fc00000), g1 = g0, rE = g0, rM = g0;
   if (okv[i]) {
@@ -1404,7 +1472,7 @@ __global__ void __launch_bounds__(128) k_start(BpParams P, int64_t n, SolveExtra
     const double rn = rint(P.n_poly);
     const HaloF h = {(float)H.c, (float)H.rvir, (float)H.rs, (float)H.mc, (float)H.phi0,
                      (float)H.GM, (float)H.M};
-    ThreadGas<float> S;
+    ThreadGas<float, W> S;
     S.c = h.c;
     S.rvir = h.rvir;
     S.rs = h.rs;
@@ -1532,6 +1600,7 @@ __global__ void __launch_bounds__(128) k_start(BpParams P, int64_t n, SolveExtra
       rM = expm1f(F_ok) * (float)((P.fb * H.M - H.Mstar) / (P.fb * H.M));
     }
   }
+  if (threadIdx.x % W) return;
   guess[i] = (double)g0;
   guess[n + i] = (double)g1;
   res32[i] = rE;
@@ -1609,13 +1678,20 @@ static int solve_launch(bp_ctx* ctx, int64_t n, const double* Mvir, const double
   int64_t blocks = (warps + SOLVE_WARPS - 1) / SOLVE_WARPS;
   bp_phase_begin(ctx, BP_PH_SOLVE);
   const int sb = bp_item_block(ctx, n, 128);
+  const bool few = n <= (int64_t)SOLVE_FEW * ctx->num_sms;  // eight threads per halo
+  const int64_t n8 = NGT * n;
+  const int sb8 = bp_item_block(ctx, n8, 128);
   k_setup<<<(unsigned)((n + sb - 1) / sb), sb, 0, ctx->stream>>>(
       ctx->p, ctx->t, n, Mvir, c, z, model, status, ctx->d_counter, X, halos, okv);
   BP_LAUNCH_CHECK(ctx, "k_setup launch");
   const double* seed = X.guess;  // the caller's starting points (or null)
   if (presolve && !(accept32 && !seed)) {
-    k_start<<<(unsigned)((n + sb - 1) / sb), sb, 0, ctx->stream>>>(ctx->p, n, X, halos, okv,
-                                                                   pguess, res32);
+    if (few)
+      k_start<NGT><<<(unsigned)((n8 + sb8 - 1) / sb8), sb8, 0, ctx->stream>>>(
+          ctx->p, n, X, halos, okv, pguess, res32);
+    else
+      k_start<1><<<(unsigned)((n + sb - 1) / sb), sb, 0, ctx->stream>>>(ctx->p, n, X, halos, okv,
+                                                                        pguess, res32);
     BP_LAUNCH_CHECK(ctx, "k_start launch");
     X.guess = pguess;
   } else if (presolve) {
@@ -1632,9 +1708,14 @@ static int solve_launch(bp_ctx* ctx, int64_t n, const double* Mvir, const double
   } else if (X.guess) {
     // starting points: the Newton from them; the halos without one get the nested iteration
     BP_CUDA(ctx, cudaMemsetAsync(okv_nested, 0, (size_t)n * sizeof(int32_t), ctx->stream));
-    k_polish<<<(unsigned)((n + sb - 1) / sb), sb, 0, ctx->stream>>>(
-        ctx->p, n, model, status, tol, ctx->d_counter, ctx->d_counter + 3, X, halos, okv,
-        okv_nested);
+    if (few)
+      k_polish<NGT><<<(unsigned)((n8 + sb8 - 1) / sb8), sb8, 0, ctx->stream>>>(
+          ctx->p, n, model, status, tol, ctx->d_counter, ctx->d_counter + 3, X, halos, okv,
+          okv_nested);
+    else
+      k_polish<1><<<(unsigned)((n + sb - 1) / sb), sb, 0, ctx->stream>>>(
+          ctx->p, n, model, status, tol, ctx->d_counter, ctx->d_counter + 3, X, halos, okv,
+          okv_nested);
     BP_LAUNCH_CHECK(ctx, "k_polish launch");
     k_solve<<<(unsigned)blocks, 32 * SOLVE_WARPS, 0, ctx->stream>>>(
         ctx->p, n, model, status, tol, ctx->d_counter, ctx->d_counter + 3, X, hpw, halos,

@@ -1,0 +1,82 @@
+"""The eight threads per halo that small catalogues get in the pre-solve and the Newton (up to 32
+halos per SM): the same bits as one thread per halo, in every mode, and less time."""
+import numpy as np
+import pytest
+import torch
+
+from tests.gpu_common import api, cuda  # noqa: F401
+
+pytestmark = pytest.mark.gpu
+N_ALL = 20000  # one thread per halo
+
+
+def _catalogue():
+    rng = np.random.default_rng(31)
+    return (10 ** rng.uniform(11.5, 15.5, N_ALL), rng.uniform(1.05, 25, N_ALL),
+            rng.uniform(0.01, 3, N_ALL), rng)
+
+
+def _seed(api, M, model, rng):
+    """Starting points near the solutions (ln r_f / r_vir, ln T r_vir / G M); some with r_f inside
+    r_vir, some missing."""
+    f = lambda k: model[api.MF[k]]
+    GM = -f("Phi0") * f("r_s") * f("m_c") / (1.0 - 1.0 / (1.0 + f("c")))
+    g = torch.stack([torch.log(f("r_f") / f("r_vir")), torch.log(f("T") * f("r_vir") / GM)])
+    g = g + cuda(rng.normal(0, 0.02, tuple(g.shape)))
+    g[0, ::11] = -0.1
+    g[:, ::17] = float("nan")
+    return g.contiguous()
+
+
+@pytest.mark.parametrize("icm", [dict(), dict(energy_sign=1), dict(Gamma=1.15), dict(Gamma=1.25)])
+@pytest.mark.parametrize("mode", ["plain", "newton", "seeded", "gated"])
+def test_same_bits(api, icm, mode):
+    M, c, z, rng = _catalogue()
+    M, c, z = cuda(M), cuda(c), cuda(z)
+    ctx = api.Context(icm=icm)
+    kw = dict(raise_on_noconv=False)
+    model, _ = ctx.solve_halos(M, c, z, **kw)
+    g = _seed(api, M, model, rng)
+
+    def solve(k):
+        a = [t[:k] for t in (M, c, z)]
+        q = g[:, :k].contiguous()
+        if mode == "plain":
+            return ctx.solve_halos(*a, **kw)
+        if mode == "newton":
+            return ctx.solve_halos_ex(*a, guess=q, max_iter=4, gate=1e-4, **kw)
+        if mode == "seeded":
+            return ctx.solve_halos_ex(*a, guess=q, seeded=True, **kw)
+        return ctx.solve_halos_ex(*a, guess=q, gate=1e-4, gated=True, **kw)
+
+    full, sf = solve(N_ALL)
+    assert int((sf == 0).sum()) > N_ALL // 2
+    for k in (1, 3, 5, 33, 1001, 4096):
+        part, sp = solve(k)
+        assert torch.equal(sp, sf[:k])
+        assert torch.equal(part.view(torch.int64), full[:, :k].contiguous().view(torch.int64))
+    torch.cuda.synchronize()
+    ctx.close()
+
+
+def test_small_catalogues_take_less_time(api):
+    """200 halos in less than 0.8 of the solve time of 15000 (0.9 with one thread per halo, 0.6 with
+    eight)."""
+    M, c, z, _ = _catalogue()
+    ctx = api.Context()
+
+    def ms(k):
+        a = [cuda(t[:k]) for t in (M, c, z)]
+        ctx.set_timing(True)
+        best = float("inf")
+        for _ in range(20):
+            ctx.phase_times()
+            ctx.solve_halos(*a, raise_on_noconv=False)
+            best = min(best, ctx.phase_times()["solve"])
+        ctx.set_timing(False)
+        return best
+
+    few, many = ms(200), ms(15000)
+    print(f"200 halos {few * 1e3:.0f} us, 15000 halos {many * 1e3:.0f} us")
+    assert few <= 0.8 * many
+    ctx.close()
