@@ -86,7 +86,9 @@ __device__ __forceinline__ void dft8(double2 (&v)[8], double2 w1, double2 w2, do
   v[6] = x6;
 }
 __device__ __forceinline__ void dft8_first(double2 (&v)[8]) {  // w = 1
-  constexpr double S = 0.70710678118654752440;
+  // e^{-i pi / 4}, one component rounded up and the other down: rounded alike, its modulus is
+  // 7e-17 above 1, which raises every power by as much
+  constexpr double SU = 0x1.6a09e667f3bcdp-1, SD = 0x1.6a09e667f3bccp-1;
 #pragma unroll
   for (int m = 0; m < 4; ++m) bfly1(v[m], v[m + 4]);
   bfly1(v[0], v[2]);
@@ -95,8 +97,8 @@ __device__ __forceinline__ void dft8_first(double2 (&v)[8]) {  // w = 1
   bflyi(v[5], v[7]);
   bfly1(v[0], v[1]);
   bflyi(v[2], v[3]);
-  bfly(v[4], v[5], make_double2(S, -S));
-  bfly(v[6], v[7], make_double2(-S, -S));
+  bfly(v[4], v[5], make_double2(SU, -SD));
+  bfly(v[6], v[7], make_double2(-SD, -SU));
   const double2 x4 = v[1], x2 = v[2], x6 = v[3], x1 = v[4], x5 = v[5], x3 = v[6];
   v[1] = x1;
   v[2] = x2;
@@ -330,7 +332,9 @@ __global__ void __launch_bounds__(BR_THREADS)
     __syncthreads();
   }
   if (t == 0) {
-    cl[b] = s_c[0] > 0 ? norm * (s_s[0] / (double)s_c[0]) : 0.0;
+    // norm times the mean in one rounding: the quotient and what it leaves
+    const double n = (double)s_c[0], q = s_s[0] / n, rest = fma(-q, n, s_s[0]) / n;
+    cl[b] = s_c[0] > 0 ? fma(norm, q, norm * rest) : 0.0;
     if (nmodes) nmodes[b] = s_c[0];
   }
 }
