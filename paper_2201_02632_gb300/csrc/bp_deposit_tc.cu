@@ -1,9 +1,9 @@
 // bp_deposit_tc.cu -- the particle deposit (Section 3.4: the separable pixel-integrated
 // kernel f_ij and the integrated SPH kernel) on the fifth-generation tensor cores.
 //
-// For one 64 x 64 pixel tile and a chunk of 64 particles k the y and b contributions are
+// For one 64 x 64 pixel tile and a slab of 16 particles k the y and b contributions are
 //   Y[j, i] += sum_k (Y_k wy_k(j)) wx_k(i),     B[j, i] += sum_k (B_k wy_k(j)) wx_k(i),
-// a rank-64 update, i.e. one 128 x 64 x 64 GEMM with the y rows and b rows stacked in M:
+// a rank-16 update, i.e. one 128 x 64 x 16 GEMM with the y rows and b rows stacked in M:
 //   A[r, k] = Y_k wy_k(r)  (r < 64),   B_k wy_k(r - 64)  (r >= 64);    Bop[i, k] = wx_k(i).
 // A cell weight is the difference of the integrated kernel at the cell's two edges, in
 // the split representation of bp_wsplit_inv (w(u) left of the particle, w(u) - 1 = -w(-u)
@@ -47,7 +47,7 @@
 //    finished tile out; the first also fetches the units, two ahead.
 // The 17 slabs (12 KB each) rotate among the warps, so a warp waits only for the MMAs 17 slabs
 // back.  What bounds it: instruction issue (72% of the issue slots used on the 4e6-particle
-// cone, 24 warps per SM; 86 warp instructions per (tile, particle) pair), the fixed-latency and
+// cone, 24 warps per SM; 104 warp instructions per (tile, particle) pair), the fixed-latency and
 // FP32-pipe stalls between them, then 10% of the producers' time waiting for a free slab.
 // Measured, k_deposit_tc on the 4e6-particle cone and on the 5e8-particle cone: 3.44 and 195.6
 // ms with two CTAs of eight warps filling K-major stages of 64 particles together (each MMA

@@ -467,7 +467,8 @@ __device__ __forceinline__ bool shrink(float* l, int& m, float& R, float n_ngb, 
 // shuffles for four particles at once.
 __global__ void __launch_bounds__(32)
     k_hsml_group(int64_t n, const float4* __restrict__ pos, const Tree tree,
-                 const uint32_t* __restrict__ ids, const float* __restrict__ R0, float n_ngb, int cap, float* h_out, uint32_t* left_k, float* left_R,
+                 const uint32_t* __restrict__ ids, const float* __restrict__ R0, float n_ngb,
+                 int cap, float* h_out, uint32_t* left_k, float* left_R,
                  unsigned long long* n_left) {
   extern __shared__ float s_dyn[];
   constexpr unsigned ALL = 0xffffffffu;
@@ -661,90 +662,90 @@ __global__ void __launch_bounds__(32)
       item = (int64_t)__shfl_sync(0xffffffffu, q, 0);
     }
     if (item >= todo) break;
-  const int64_t k = left_k ? left_k[item] : item;
-  const float4 p = pos[k];
-  const float3 pc = make_float3(p.x, p.y, p.z);
-  const uint32_t id = ids[k];
-  float R = left_k ? left_R[item] : R0[k];
-  float r_short = 0.f, r_over = INFINITY;  // N_eff too small at r_short; too many at r_over
-  float cut = 0.63f;  // next cut of a radius with far too many particles
-  float h = __int_as_float(0x7fc00000);
-  bool done = false;
-  for (int round = 0; round < HS_MAX_ROUNDS && !done; ++round) {
-    const float R2 = R * R;
-    // the particles within R, in tree order
-    uint32_t off = 0;
-    search(tree, pc, pc, R2, lane, [&](uint32_t node, unsigned hits, const float4&, const float4&) {
-      while (hits) {  // four leaves at a time: their loads overlap
-        float d2[4];
-#pragma unroll
-        for (int q = 0; q < 4; ++q) {
-          d2[q] = INFINITY;
-          if (hits) d2[q] = dist2(pos[((uint64_t)node * 32 + __ffs(hits) - 1) * 32 + lane], p);
-          hits &= hits - 1;
+    const int64_t k = left_k ? left_k[item] : item;
+    const float4 p = pos[k];
+    const float3 pc = make_float3(p.x, p.y, p.z);
+    const uint32_t id = ids[k];
+    float R = left_k ? left_R[item] : R0[k];
+    float r_short = 0.f, r_over = INFINITY;  // N_eff too small at r_short; too many at r_over
+    float cut = 0.63f;  // next cut of a radius with far too many particles
+    float h = __int_as_float(0x7fc00000);
+    bool done = false;
+    for (int round = 0; round < HS_MAX_ROUNDS && !done; ++round) {
+      const float R2 = R * R;
+      // the particles within R, in tree order
+      uint32_t off = 0;
+      search(tree, pc, pc, R2, lane, [&](uint32_t node, unsigned hits, const float4&, const float4&) {
+        while (hits) {  // four leaves at a time: their loads overlap
+          float d2[4];
+  #pragma unroll
+          for (int q = 0; q < 4; ++q) {
+            d2[q] = INFINITY;
+            if (hits) d2[q] = dist2(pos[((uint64_t)node * 32 + __ffs(hits) - 1) * 32 + lane], p);
+            hits &= hits - 1;
+          }
+  #pragma unroll
+          for (int q = 0; q < 4; ++q) {
+            const bool in = d2[q] < R2;
+            const unsigned m = __ballot_sync(0xffffffffu, in);
+            const uint32_t at = off + __popc(m & ((1u << lane) - 1u));
+            if (in && at < (uint32_t)cap) buf[at] = d2[q];
+            off += __popc(m);
+          }
         }
-#pragma unroll
-        for (int q = 0; q < 4; ++q) {
-          const bool in = d2[q] < R2;
-          const unsigned m = __ballot_sync(0xffffffffu, in);
-          const uint32_t at = off + __popc(m & ((1u << lane) - 1u));
-          if (in && at < (uint32_t)cap) buf[at] = d2[q];
-          off += __popc(m);
+        return off <= (uint32_t)(HS_SCAN_CAPS * cap);
+      });
+      __syncwarp();
+      if (off > (uint32_t)(HS_SCAN_CAPS * cap)) {  // far too many: try a smaller radius first
+        const float Rn = (r_short > 0.f ? 0.63f : cut) * R;
+        if (Rn > r_short) {  // (how many is not known: the cuts get deeper until one is too deep)
+          cut = fmaxf(cut * cut, 0.02f);
+          R = Rn;
+          __syncwarp();
+          continue;
         }
       }
-      return off <= (uint32_t)(HS_SCAN_CAPS * cap);
-    });
-    __syncwarp();
-    if (off > (uint32_t)(HS_SCAN_CAPS * cap)) {  // far too many: try a smaller radius first
-      const float Rn = (r_short > 0.f ? 0.63f : cut) * R;
-      if (Rn > r_short) {  // (how many is not known: the cuts get deeper until one is too deep)
-        cut = fmaxf(cut * cut, 0.02f);
-        R = Rn;
+      // too many candidates: shrink towards the last short radius while that bracket is wide,
+      // else stream the sums over the cube at this radius
+      const bool stream = off > (uint32_t)cap;
+      if (stream && !(r_short > 0.f && R <= 1.3f * r_short) && round < HS_MAX_ROUNDS - 8) {
+        r_over = R;
+        R = fmaxf(r_short, R * cbrtf(0.5f * cap / (float)off));
+        if (!(R > r_short)) R = 0.5f * (r_short + r_over);
+        continue;
+      }
+      const int total = (int)off;
+      float f, df;
+      if (stream) neff_stream(tree, pos, p, R, R, lane, f, df);
+      else neff<true>(buf, total, R, lane, f, df);
+      if (f < n_ngb) {  // not enough within R: grow
+        r_short = R;
+        float grow = 1.1f * cbrtf(n_ngb / fmaxf(f, 1e-3f));
+        grow = fminf(fmaxf(grow, 1.15f), 4.0f);
+        R = fminf(R * grow, 0.5f * (R + r_over));
+        if (!(R > r_short)) R = r_short * 1.15f;
         __syncwarp();
         continue;
       }
-    }
-    // too many candidates: shrink towards the last short radius while that bracket is wide,
-    // else stream the sums over the cube at this radius
-    const bool stream = off > (uint32_t)cap;
-    if (stream && !(r_short > 0.f && R <= 1.3f * r_short) && round < HS_MAX_ROUNDS - 8) {
-      r_over = R;
-      R = fmaxf(r_short, R * cbrtf(0.5f * cap / (float)off));
-      if (!(R > r_short)) R = 0.5f * (r_short + r_over);
-      continue;
-    }
-    const int total = (int)off;
-    float f, df;
-    if (stream) neff_stream(tree, pos, p, R, R, lane, f, df);
-    else neff<true>(buf, total, R, lane, f, df);
-    if (f < n_ngb) {  // not enough within R: grow
-      r_short = R;
-      float grow = 1.1f * cbrtf(n_ngb / fmaxf(f, 1e-3f));
-      grow = fminf(fmaxf(grow, 1.15f), 4.0f);
-      R = fminf(R * grow, 0.5f * (R + r_over));
-      if (!(R > r_short)) R = r_short * 1.15f;
-      __syncwarp();
-      continue;
-    }
-    // N_eff(R) >= n_ngb: the root in (0, R]
-    h = R;
-    if (f - n_ngb >= 1e-6f * n_ngb) {
-      float lo = 0.f, hi = R, step = INFINITY;
-      float x = fminf(R, fmaxf(0.5f * R, R * cbrtf(n_ngb / f)));
-      for (int it = 0; it < 40; ++it) {
-        if (stream) neff_stream(tree, pos, p, R, x, lane, f, df);
-        else neff<false>(buf, total, x, lane, f, df);
-        if (!newton(n_ngb, f, df, x, lo, hi, h, step)) break;
+      // N_eff(R) >= n_ngb: the root in (0, R]
+      h = R;
+      if (f - n_ngb >= 1e-6f * n_ngb) {
+        float lo = 0.f, hi = R, step = INFINITY;
+        float x = fminf(R, fmaxf(0.5f * R, R * cbrtf(n_ngb / f)));
+        for (int it = 0; it < 40; ++it) {
+          if (stream) neff_stream(tree, pos, p, R, x, lane, f, df);
+          else neff<false>(buf, total, x, lane, f, df);
+          if (!newton(n_ngb, f, df, x, lo, hi, h, step)) break;
+        }
       }
+      done = true;
+      __syncwarp();
     }
-    done = true;
+    if (lane == 0) {
+      h_out[id] = done ? h : __int_as_float(0x7fc00000);
+      if (!done) atomicAdd((unsigned long long*)nfail, 1ull);
+    }
     __syncwarp();
-  }
-  if (lane == 0) {
-    h_out[id] = done ? h : __int_as_float(0x7fc00000);
-    if (!done) atomicAdd((unsigned long long*)nfail, 1ull);
-  }
-  __syncwarp();
   }
 }
 
@@ -873,8 +874,8 @@ extern "C" int bp_smoothing_lengths(bp_ctx* ctx, int64_t n, const float* x, cons
     blocks = std::min(blocks, (int64_t)ctx->num_sms * 26);  // (they fetch their particles)
   }
   k_hsml<<<bp_item_grid(blocks), 32, smem, ctx->stream>>>(
-      n, pos, tree, E, (float)n_ngb, cap, (const float*)F, left_k, left_R, n_left, n_left + 1, h_out,
-      ctx->d_counter + 5);
+      n, pos, tree, E, (float)n_ngb, cap, (const float*)F, left_k, left_R, n_left, n_left + 1,
+      h_out, ctx->d_counter + 5);
   BP_LAUNCH_CHECK(ctx, "smoothing lengths");
   BP_CUDA(ctx, cudaMemcpyAsync(ctx->h_pinned + 5, ctx->d_counter + 5, sizeof(int64_t),
                                cudaMemcpyDeviceToHost, ctx->stream));

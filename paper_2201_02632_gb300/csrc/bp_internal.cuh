@@ -78,7 +78,7 @@ struct PpPrepared {
   bp_map_geom g;
   int select, ts, unit;
   int ks;  // class bits of the keys below the tile
-  int64_t np, n_tiles, n_keys, max_units, n_slots;
+  int64_t np, n_tiles, max_units, n_slots;
   const uint32_t* vals;
   int64_t *tstart, *uoff, *soff;
   void* units;

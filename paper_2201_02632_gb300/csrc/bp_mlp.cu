@@ -61,8 +61,9 @@ __device__ __forceinline__ float gelu_grad(float x) {
 constexpr int MT_ROWS = 32, MT_THREADS = 256;
 // Tiles whose weight gradients are added up in registers before they go into the CTA's partials:
 // one chain of FP32 additions over all of a CTA's rows loses bits as its root (4e6 rows, terms of
-// random sign: 4.1e-6 relative, 6.8e-7 with this, at 18.0 instead of 16.9 ms).  512 rows are fewer additions in a row
-// than the 256 rows and then n / 256 partials of gradients formed in chunks, for every n.
+// random sign: 4.1e-6 relative, 6.8e-7 with this, at 18.0 instead of 16.9 ms).  512 rows are fewer
+// additions in a row than the 256 rows and then n / 256 partials of gradients formed in chunks, for
+// every n.
 constexpr int MT_FOLD = 16;
 constexpr int LDW = HID + 4;  // padded row length in shared memory
 

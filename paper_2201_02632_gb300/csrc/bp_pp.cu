@@ -341,7 +341,10 @@ __global__ void __launch_bounds__(ASSIGN_THREADS) k_assign4(AssignArgs a, BpTabl
 // 16 particles without y), SMALL_KS with the small-particle deposit on as well.  The extra bit
 // keeps the full-scale sort at two digits (16 bits); the deposit gains more than the sort
 // loses: 5e8-particle cone 140.4 -> 134.4 ms against 25.9 -> 28.7 ms, 4e6-particle cone 2.54 ->
-// 2.39 ms against 0.29 -> 0.33 ms.
+// 2.39 ms against 0.29 -> 0.33 ms.  Where it brings a third digit (4097 to 8192 tiles), three of
+// six bits sort as fast as two of eight: 5120^2, 2e8 particles, without and with the bit: sort 4.64
+// and 4.53 ms, deposit 16.0 and 15.5 ms.  Where it brings a second (129 to 256 tiles), it costs 20
+// to 30 us: 1e6 particles on 832^2, no gain in the deposit, 396 and 416 us.
 constexpr int KS_FIELD = 1, SMALL_KS = 4;
 // Large-particle keys of a tile (its first ones)
 __host__ __device__ __forceinline__ int large_keys(int ks) { return ks ? 2 : 1; }
@@ -1010,8 +1013,8 @@ int prepare_units(bp_ctx* ctx, const uint32_t* keys, const uint32_t* vals, int64
                   int64_t n_tiles, PpPrepared* P, int ks = 0) {
   int r;
   const int64_t n_keys = n_tiles << ks;
-  // particles per work unit: the context's value, or (auto) about 16 units per
-  // resident CTA, at least 2048
+  // particles per work unit: the context's value, or (auto) about 32 units per SM (the
+  // tensor-core deposit holds one CTA per SM, the SIMT one two), at least 2048
   int64_t unit64 = ctx->pp_unit;
   if (unit64 <= 0) {
     unit64 = np / ((int64_t)ctx->num_sms * 2 * 16);
@@ -1048,7 +1051,6 @@ int prepare_units(bp_ctx* ctx, const uint32_t* keys, const uint32_t* vals, int64
   P->unit = unit;
   P->np = np;
   P->n_tiles = n_tiles;
-  P->n_keys = n_keys;
   P->ks = ks;
   P->max_units = max_units;
   P->n_slots = ctx->h_pinned[1];

@@ -16,9 +16,10 @@
 // Kernels: k_setup (the scalar set-up, one thread per halo), k_start (the reduced problem in
 // FP32 to its rounding floor: starting points; one thread per halo, eight in small catalogues),
 // k_polish (FP64: a two-dimensional Newton in (ln T, ln r_f) from the starting point, one
-// quadrature per step, to the tolerance; threads as k_start), k_solve (the nested iteration, a warp per halo, for halos
-// without a starting point), then k_setup + k_solve again, nested, for halos the Newton did not
-// bring in (the fallback).  BP_SOLVE_FP32_GATED: k_presolve or k_start, then k_accept32.
+// quadrature per step, to the tolerance; threads as k_start), k_solve (the nested iteration, a
+// warp per halo, for halos without a starting point), then k_setup + k_solve again, nested, for
+// halos the Newton did not bring in (the fallback).  BP_SOLVE_FP32_GATED: k_presolve or k_start,
+// then k_accept32.
 #include <algorithm>
 #include <vector>
 
@@ -202,9 +203,9 @@ struct Sums {
   double Im, In, Ip, Jm, Jn;  // int theta^{n-1,n,n+1} r^2, int theta^{n-1,n} Phi r^2
 };
 
-// W lanes per halo (32: a warp; 16: two halos per warp), NG Gauss-Legendre points per panel
-template <int W, int NG>
-struct SolverT {
+// A warp per halo
+struct Solver {
+  static constexpr int W = 32, NG = NGL;  // lanes per halo, Gauss-Legendre points per panel
   static constexpr int NS = (MAX_PANEL_A * NG + W - 1) / W;  // slots per lane
   const Halo& h;
   double n;     // polytropic index
@@ -218,12 +219,10 @@ struct SolverT {
   int a_cnt, f_cnt;  // slots in use (the nodes of a lane fill slots 0 .. cnt - 1)
   bool full_a;  // r_f >= r_vir: region A is complete and region B follows
 
-  __device__ SolverT(const Halo& hh, double nn) : h(hh), n(nn) {
+  __device__ Solver(const Halo& hh, double nn) : h(hh), n(nn) {
     double rn = rint(nn);
     n_int = (fabs(nn - rn) < 1e-12 && rn >= 1 && rn <= 16) ? (int)rn : -1;
   }
-  __device__ static double glx(int j) { return NG == NGL ? c_glx[j] : c_glx8[j]; }
-  __device__ static double glw(int j) { return NG == NGL ? c_glw[j] : c_glw8[j]; }
   // sum over the W lanes of this halo (xor butterflies stay inside aligned groups of W)
   __device__ static double group_sum(double v) {
     for (int o = W / 2; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
@@ -267,8 +266,8 @@ struct SolverT {
       phi[t] = h.phi0;
       if (q >= MAX_PANEL_A * NG || !panel_a(p, xa, h.rs, a, b)) continue;
       double mid = 0.5 * (a + b), hw = 0.5 * (b - a);
-      double r = mid + hw * glx(j);
-      r2w[t] = hw * glw(j) * r * r;
+      double r = mid + hw * c_glx[j];
+      r2w[t] = hw * c_glw[j] * r * r;
       phi[t] = phi_of(h, r);
       cnt = t + 1;
     }
@@ -295,8 +294,8 @@ struct SolverT {
       if (!(a < rf)) continue;
       const double b = fmin(2.0 * a, rf);
       double mid = 0.5 * (a + b), hw = 0.5 * (b - a);
-      double r = mid + hw * glx(j);
-      f_r2w[t] = hw * glw(j) * r * r;
+      double r = mid + hw * c_glx[j];
+      f_r2w[t] = hw * c_glw[j] * r * r;
       f_phi[t] = -h.GM / r;
       f_cnt = t + 1;
     }
@@ -333,7 +332,6 @@ struct SolverT {
     return s;
   }
 };
-using Solver = SolverT<32, NGL>;
 
 // Reduced problem at a given r_f: T from the gas-mass condition.
 struct Eval {
@@ -1152,7 +1150,7 @@ __global__ void __launch_bounds__(128) k_polish(
 // Starting points for the FP64 solve: the same reduced problem (T from the gas-mass
 // condition at each r_f, Newton in ln r_f on the energy condition) in FP32, to
 // residuals of about 1e-4 (FP32 runs at many times the FP64 rate on this GPU).  The
-// FP64 two-dimensional Newton of k_solve then takes the starting point to the
+// FP64 two-dimensional Newton (k_polish) then takes the starting point to the
 // tolerance; a halo the pre-solve cannot bring in gets no starting point (NaN) and the
 // full FP64 iteration.
 struct HaloF {
@@ -1180,9 +1178,9 @@ struct SumsF {
   float Im, In, Ip, Jm, Jn;
 };
 
-// FP32 counterpart of SolverT: the same panels and node slots (W lanes, NG points)
-template <int W, int NG>
-struct SolverFT {
+// FP32 counterpart of Solver: the same panels, 8 points each
+struct SolverF {
+  static constexpr int W = 32, NG = NGL_PRE;
   static constexpr int NS = (MAX_PANEL_A * NG + W - 1) / W;
   const HaloF& h;
   int n_int;
@@ -1191,7 +1189,7 @@ struct SolverFT {
   int a_cnt, f_cnt;
   bool full_a;
 
-  __device__ SolverFT(const HaloF& hh, float nn, int ni) : h(hh), n_int(ni), n(nn) {}
+  __device__ SolverF(const HaloF& hh, float nn, int ni) : h(hh), n_int(ni), n(nn) {}
   static_assert(NG == NGL_PRE, "FP32 rule tabulated for NGL_PRE points only");
   __device__ static float glx(int j) { return c_glxf[j]; }
   __device__ static float glw(int j) { return c_glwf[j]; }
@@ -1297,7 +1295,6 @@ struct SolverFT {
   }
 };
 
-using SolverF = SolverFT<32, NGL_PRE>;
 
 // guess[i] = ln(r_f / r_vir), guess[n + i] = ln(T r_vir / (G M)), or NaN
 __global__ void __launch_bounds__(32 * SOLVE_WARPS) k_presolve(
@@ -1452,12 +1449,13 @@ __global__ void __launch_bounds__(32 * SOLVE_WARPS) k_presolve(
 }
 
 // The pre-solve of every mode but the gated one without a seed: the same iteration as k_presolve,
-// W threads per halo (as k_polish) with the tabulated nodes (no shuffles, no scalar work repeated in 32
-// lanes, no logarithm per node).  A warp runs as long as its slowest halo.  Measured from the
-// default start: 1e6 halos 1.4 ms (k_presolve: 11.2 ms).  It sums in another order than
-// k_presolve, which moves the FP32 solutions within their rounding floor (1e-6 relative); the
-// gated mode without a seed returns those solutions as its answer and keeps k_presolve, so that
-// its results stay what they are.
+// W threads per halo (as k_polish) with the tabulated nodes (no logarithm per node; one thread:
+// no shuffles, no scalar work repeated in 32 lanes).  A warp runs as long as its slowest halo.
+// Measured with one thread from the default start: 1e6 halos 1.4 ms (k_presolve: 11.2 ms).  It
+// sums in another order than k_presolve, which moves the FP32 solutions within their rounding
+// floor (1e-6 relative); the gated mode without a seed returns those solutions as its answer and
+// keeps k_presolve, so that its results stay what they are (above 1e4 halos the FP64 solve is
+// now the faster of the two: 2e5 halos 1.8 and 3.2 ms).
 template <int W>
 __global__ void __launch_bounds__(128) k_start(BpParams P, int64_t n, SolveExtra X,
                                                const Halo* __restrict__ halos,
