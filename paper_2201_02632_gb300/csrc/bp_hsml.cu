@@ -337,10 +337,11 @@ __device__ __forceinline__ void neff_quarter(float* l, int len, int steps, float
 }
 
 // one Newton step on ln N_eff(ln h) = ln n_ngb (nearly linear) from x inside the bisection
-// bracket [lo, hi]; h: the answer so far; step: the last step's length (infinite at first);
-// false: it is the last.  A step that is not half as long as the last is a bisection: with a clump
-// between x and the root, Newton can jump to and fro between its two sides, both within the
-// bracket, for ever (light-cone particles, N_ngb = 200: 3 in 1e5).
+// bracket [lo, hi]; h: the answer so far; step: the length of the last step if it was one of
+// Newton's, else infinite (as at first); false: this step is the last.  A step that is not half as
+// long as Newton's last becomes a bisection: with a clump between x and the root, Newton can jump
+// to and fro between its two sides, both within the bracket, for ever (light-cone particles, N_ngb
+// = 200: 3 in 1e5).  The bracket includes its ends: a step that rounds to none has converged.
 __device__ __forceinline__ bool newton(float n_ngb, float f, float df, float& x, float& lo,
                                        float& hi, float& h, float& step) {
   const float F = f - n_ngb;
@@ -348,12 +349,13 @@ __device__ __forceinline__ bool newton(float n_ngb, float f, float df, float& x,
   h = x;
   if (fabsf(F) <= 1e-6f * n_ngb) return false;
   float xn = (df > 0.f) ? x * __expf(__logf(n_ngb / f) * f / (x * df)) : 0.f;
-  const bool in = xn > lo && xn < hi && fabsf(xn - x) < 0.5f * step;
+  const bool in = xn >= lo && xn <= hi && fabsf(xn - x) < 0.5f * step && xn > 0.f;
   if (!in) xn = 0.5f * (lo + hi);
-  step = fabsf(xn - x);
+  const float s = fabsf(xn - x);
+  step = in ? s : INFINITY;
   // what a Newton step leaves is of the order of its square; next to it the FP32 sums' rounding
   // is the larger part (stopping at 1e-6 instead leaves the same errors, at 0.6 more steps)
-  const bool last = step <= (in ? 2e-4f : 1e-6f) * x || hi - lo <= 1e-6f * hi;
+  const bool last = s <= (in ? 2e-4f : 1e-6f) * x || hi - lo <= 1e-6f * hi;
   h = x = xn;
   return !last;
 }

@@ -79,3 +79,25 @@ def test_far_too_large_guesses_cost_little(api, ctx):
 
     none, far = ms(None), ms(1000.0 * h)
     assert far <= 5.0 * none, (far, none)
+
+
+def test_residuals_of_clustered_particles(api, ctx):
+    """N_eff(h) of every particle, in FP64.  h is an FP32 number: 6e-8 of it times the slope
+    d ln N_eff / d ln h, which reaches 30 with a halo at the kernel's edge, is 2e-6 of N_eff; the
+    FP32 sums add 1e-6, the solve's stop 1e-6: 5e-6.  (1e-5 where the end of a solve was found by
+    halving a bracket down to 1e-6 of h.)"""
+    n, n_ngb = 120000, 100.0
+    x = [cuda(v) for v in _cone(n)]
+    h = ctx.smoothing_lengths(*x, n_ngb).double()
+    p = torch.stack(x, 1).double()
+    worst = 0.0
+    for a in range(0, n, 1000):
+        d = torch.zeros((min(1000, n - a), n), dtype=torch.float64, device="cuda")
+        for k in range(3):
+            d += (p[a:a + 1000, k, None] - p[None, :, k]) ** 2
+        u = (1.0 - d.sqrt_() / h[a:a + 1000, None]).clamp_(min=0.0)
+        v = (u - 0.5).clamp(min=0.0)
+        eff = 32.0 / 3.0 * (2.0 * u ** 3 - 8.0 * v ** 3).sum(1)
+        worst = max(worst, float((eff / n_ngb - 1.0).abs().max()))
+    print(f"worst |N_eff / N_ngb - 1| {worst:.1e}")
+    assert worst <= 5e-6
