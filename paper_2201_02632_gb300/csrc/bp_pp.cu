@@ -1440,7 +1440,8 @@ int bp_pp_deposit(bp_ctx* ctx, int64_t n, const float* assigned, const bp_map_ge
   const PpPrepared& P = ctx->pp_prep;
   if (!P.valid || P.assigned != assigned || P.n != n || !geom || P.select != select ||
       P.ts != ctx->pp_tile || memcmp(&P.g, geom, sizeof(bp_map_geom)) != 0 ||
-      (P.np > 0 && P.ks != pp_class_bits(ctx, P.ts, pp_small_span(ctx, P.ts, geom))))
+      // (either deposit kernel takes a list with or without the field bit)
+      (P.np > 0 && (P.ks == SMALL_KS) != (pp_small_span(ctx, P.ts, geom) > 0)))
     return bp_fail(ctx, BP_EINVAL, "bp_pp_deposit: no bp_pp_prepare of these records");
   if (P.np == 0 || n == 0) return BP_OK;
   for (int k : {(int)WS_KEYS0, (int)WS_VALS0, (int)WS_KEYS1, (int)WS_VALS1, (int)WS_TILES,
