@@ -264,45 +264,84 @@ __global__ void __launch_bounds__(Fft<LG>::T* Fft<LG>::F, Fft<LG>::N <= 4096 ? 2
   for (int m = 0; m < P::E; ++m) v[m] = in[(int64_t)kx * N + j + m * T];
   // |l|^2 = c2 ((kx / Lx)^2 + (ky / Ly)^2), every operation rounded as written; it does not
   // decrease with |ky|
-  for (int q = threadIdx.x; q < F * (nb + 1); q += blockDim.x) {
-    const int ff = q / (nb + 1), b = q % (nb + 1);
-    const int k = min(col0 + ff, ncol - 1);
-    const int fx = k < nx / 2 ? k : k - nx;
+  auto kx2 = [&](int ff) {
+    const int k = min(col0 + ff, ncol - 1), fx = k < nx / 2 ? k : k - nx;
     const double ux = __dmul_rn((double)fx, inv_lx);
-    const double ux2 = __dmul_rn(ux, ux), e2 = E.e2[b];
+    return __dmul_rn(ux, ux);
+  };
+  auto l2 = [&](double ux2, int ky) {
+    const double uy = __dmul_rn((double)ky, inv_ly);
+    return __dmul_rn(c2, __dadd_rn(ux2, __dmul_rn(uy, uy)));
+  };
+  if constexpr (F > 1) {  // short columns: every |l|^2 once, in the transforms' arrays
+    for (int q = threadIdx.x; q < F * (N / 2 + 1); q += blockDim.x) {
+      const int ff = q / (N / 2 + 1), k = q % (N / 2 + 1);
+      s_d[(size_t)ff * 2 * P::PADN + k] = l2(kx2(ff), k);
+    }
+    __syncthreads();
+  }
+  // every (column, b) with b < n, a thread each (no divisions)
+  auto each = [&](int n, auto&& fn) {
+    for (int ff = 0, b = threadIdx.x;; b += blockDim.x) {
+      for (; b >= n; b -= n)
+        if (++ff == F) return;
+      fn(ff, b);
+    }
+  };
+  each(nb + 1, [&](int ff, int b) {
+    const double ux2 = F > 1 ? 0.0 : kx2(ff), e2 = E.e2[b];
+    const double* s_l = s_d + (size_t)ff * 2 * P::PADN;
     int lo = 0, hi = N / 2 + 1;  // the answer is in [lo, hi]
     while (lo < hi) {
       const int mid = (lo + hi) >> 1;
-      const double uy = __dmul_rn((double)mid, inv_ly);
-      if (__dmul_rn(c2, __dadd_rn(ux2, __dmul_rn(uy, uy))) >= e2) hi = mid; else lo = mid + 1;
+      if ((F > 1 ? s_l[mid] : l2(ux2, mid)) >= e2) hi = mid; else lo = mid + 1;
     }
     s_f[ff][b] = (short)lo;
-  }
+  });
+  if constexpr (F > 1) __syncthreads();
   P::run(v, j, re, im, tw);
   __syncthreads();
 #pragma unroll
   for (int m = 0; m < P::E; ++m)
     re[P::at(j + m * T)] = fma(v[m].x, v[m].x, v[m].y * v[m].y);
   __syncthreads();
-  // a warp per (column, bin): |ky| in its range, ky and -ky (one mode at 0 and at N / 2)
-  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
-  for (int q = wid; q < F * nb; q += nw) {
-    const int ff = q / nb, b = q % nb;
-    if (col0 + ff >= ncol) continue;
-    const double* p = s_d + (size_t)ff * 2 * P::PADN;
+  // |ky| in the bin's range, ky and -ky (one mode at 0 and at N / 2)
+  auto put = [&](int ff, int b, double s) {
     const int k0 = s_f[ff][b], k1 = s_f[ff][b + 1];
+    const int k = col0 + ff, w = k > 0 && k < nx / 2 ? 2 : 1;
+    const int ends = (k0 == 0 && k1 > 0 ? 1 : 0) + (k0 <= N / 2 && k1 > N / 2 ? 1 : 0);
+    psum[(int64_t)k * nb + b] = w * s;
+    pcnt[(int64_t)k * nb + b] = w * (2 * (k1 - k0) - ends);
+  };
+  // Short columns, several per CTA: a thread per (column, bin), Kahan sums.  (A warp each left two
+  // warps 960 turns at 64 columns and 30 bins.  A map of 512 x 2: 482 us before, 47 now; 512 x 128
+  // with 256 bins: 310 and 53 us.)
+  if constexpr (F > 1) {
+    each(nb, [&](int ff, int b) {
+      if (col0 + ff >= ncol) return;
+      const double* p = s_d + (size_t)ff * 2 * P::PADN;
+      double s = 0.0, c = 0.0;
+      for (int k = s_f[ff][b]; k < s_f[ff][b + 1]; ++k) {
+        const double v = p[P::at(k)] + (k > 0 && k < N / 2 ? p[P::at(N - k)] : 0.0);
+        const double y = v - c, t = s + y;
+        c = (t - s) - y;
+        s = t;
+      }
+      put(ff, b, s);
+    });
+    return;
+  }
+  // a warp per bin
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
+  for (int b = wid; b < nb; b += nw) {
+    const int k0 = s_f[0][b], k1 = s_f[0][b + 1];
     double s = 0.0;
     for (int k = k0 + lane; k < k1; k += 32) {
-      s += p[P::at(k)];
-      if (k > 0 && k < N / 2) s += p[P::at(N - k)];
+      s += s_d[P::at(k)];
+      if (k > 0 && k < N / 2) s += s_d[P::at(N - k)];
     }
     for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-    if (lane == 0) {
-      const int k = col0 + ff, w = k > 0 && k < nx / 2 ? 2 : 1;
-      const int ends = (k0 == 0 && k1 > 0 ? 1 : 0) + (k0 <= N / 2 && k1 > N / 2 ? 1 : 0);
-      psum[(int64_t)k * nb + b] = w * s;
-      pcnt[(int64_t)k * nb + b] = w * (2 * (k1 - k0) - ends);
-    }
+    if (lane == 0) put(0, b, s);
   }
 }
 
