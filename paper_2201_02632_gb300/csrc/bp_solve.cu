@@ -522,9 +522,11 @@ __device__ bool halo_setup(const BpParams& P, const BpTables& TB, int64_t n, int
 constexpr int SOLVE_WARPS = 4;  // warps per block
 // Halos per SM up to which k_start and k_polish take eight threads a halo: one thread per halo is a
 // long serial chain that a small catalogue cannot hide, eight threads repeat the scalar part.  The
-// whole solve with eight threads and with one: 40 halos 195 and 266 us, 1000 halos 206 and 298,
-// 3000 halos 245 and 336, 6000 halos (39 per SM) 321 and 311, 2e4 halos 645 and 423 us.
-constexpr int SOLVE_FEW = 32;
+// whole solve with eight threads and with one: 40 halos 195 and 266 us, 1000 halos 212 and 301,
+// 3000 halos 250 and 339, 6000 halos (39 per SM) 312 and 313, 2e4 halos 633 and 425 us.  With a
+// polytropic index that is no integer the nodes' powers are most of the work (Gamma = 1.15: 300
+// halos 298 and 697 us, 1e4 (66 per SM) 654 and 750, 1.5e4 (99 per SM) 872 and 782 us).
+constexpr int SOLVE_FEW = 32, SOLVE_FEW_POW = 80;
 // |R_e| below which the nested iteration hands over to the two-dimensional Newton
 constexpr double NEWTON2D_SWITCH = 1e-3;
 
@@ -842,7 +844,8 @@ struct Sums3 {
 };
 __device__ __forceinline__ double t_log1p(double x) { return log1p(x); }
 __device__ __forceinline__ float t_log1p(float x) { return log1pf(x); }
-__device__ __forceinline__ double t_pow(double x, double y) { return pow(x, y); }
+// x in (0, 1], |y ln x| at most 30: to 3e-15 of pow, at half its FP64 operations
+__device__ __forceinline__ double t_pow(double x, double y) { return exp(y * log(x)); }
 __device__ __forceinline__ float t_pow(float x, float y) { return powf(x, y); }
 __device__ __forceinline__ double t_fma(double x, double y, double z) { return __fma_rn(x, y, z); }
 __device__ __forceinline__ float t_fma(float x, float y, float z) { return __fmaf_rn(x, y, z); }
@@ -937,17 +940,19 @@ struct ThreadGas {
     return p;
   }
   __device__ void init() { nfull = cut(c, cg, cw); }
-  // Panel p of region B (p < MAX_PANEL_B, its start below r_f): its sums, returns its half width
-  __device__ __forceinline__ Real panel_b(int p, Real rf, Real t0, Real t1, Sums3<Real>& v) const {
+  // Panel p of region B (p < MAX_PANEL_B, its start below r_f): middle and half width, and node j's
+  // weight and theta = t0 + t1 / r
+  __device__ __forceinline__ void span_b(int p, Real rf, Real& mid, Real& hw) const {
     const Real a = rvir * (Real)(1 << p);
     const Real b = (Real)2 * a < rf ? (Real)2 * a : rf;
-    const Real mid = (Real)0.5 * (a + b), hw = (Real)0.5 * (b - a);
-#pragma unroll
-    for (int j = 0; j < NGT; ++j) {
-      const Real r = t_fma(hw, tab_x8(Real(), j), mid);
-      acc(v, t_mul(t_mul(tab_w8(Real(), j), r), r), t0 + t1 / r);
-    }
-    return hw;
+    mid = (Real)0.5 * (a + b);
+    hw = (Real)0.5 * (b - a);
+  }
+  __device__ __forceinline__ static void node_b(Real mid, Real hw, int j, Real t0, Real t1, Real& w,
+                                                Real& th) {
+    const Real r = t_fma(hw, tab_x8(Real(), j), mid);
+    w = t_mul(t_mul(tab_w8(Real(), j), r), r);
+    th = t0 + t1 / r;
   }
   // Integrals over [0, rf] with theta = 1 + (Phi0 - Phi) inv_n1T
   __device__ Sums3<Real> integrals(Real rf, Real inv_n1T) const {
@@ -977,7 +982,14 @@ struct ThreadGas {
       if (full) {
         for (int p = 0; p < MAX_PANEL_B && rvir * (Real)(1 << p) < rf; ++p) {
           Sums3<Real> v = {0, 0, 0};
-          const Real hw = panel_b(p, rf, t0, t1, v);
+          Real mid, hw;
+          span_b(p, rf, mid, hw);
+#pragma unroll
+          for (int j = 0; j < NGT; ++j) {
+            Real w, th;
+            node_b(mid, hw, j, t0, t1, w, th);
+            acc(v, w, th);
+          }
           add(s, v, hw);
         }
       }
@@ -987,19 +999,23 @@ struct ThreadGas {
         for (int p = 0; p < MAX_PANEL_B && rvir * (Real)(1 << p) < rf; ++p) ++nt;
       for (int p0 = 0; p0 < nt; p0 += W) {
         const int p = p0 + at();
+        const bool in_b = p > np && p < nt;
+        Real mid = 0, hw = 0;
+        if (in_b) span_b(p - np - 1, rf, mid, hw);
+        const int k = (p < np ? p : 0) * NGT;
         Sums3<Real> v = {0, 0, 0};
-        Real f = rs3;
-        if (p <= np) {
-          const int k = (p < np ? p : 0) * NGT;
 #pragma unroll
-          for (int j = 0; j < NGT; ++j) {
-            const Real w = p < np ? tab_w(Real(), k + j) : full ? cw[j] : w2[j];
-            const Real g = p < np ? tab_g(Real(), k + j) : full ? cg[j] : g2[j];
-            acc(v, w, t_fma(-q, g, (Real)1));
+        for (int j = 0; j < NGT; ++j) {  // the powers in one place for the panels of both regions
+          Real w = 0, th = 1;
+          if (in_b) {
+            node_b(mid, hw, j, t0, t1, w, th);
+          } else if (p <= np) {
+            w = p < np ? tab_w(Real(), k + j) : full ? cw[j] : w2[j];
+            th = t_fma(-q, p < np ? tab_g(Real(), k + j) : full ? cg[j] : g2[j], (Real)1);
           }
-        } else if (p < nt) {
-          f = panel_b(p - np - 1, rf, t0, t1, v);
+          acc(v, w, th);
         }
+        const Real f = in_b ? hw : rs3;
         __syncwarp(group());
         for (int k = 0; k < W && p0 + k < nt; ++k) {
           Sums3<Real> u;
@@ -1676,7 +1692,10 @@ static int solve_launch(bp_ctx* ctx, int64_t n, const double* Mvir, const double
   int64_t blocks = (warps + SOLVE_WARPS - 1) / SOLVE_WARPS;
   bp_phase_begin(ctx, BP_PH_SOLVE);
   const int sb = bp_item_block(ctx, n, 128);
-  const bool few = n <= (int64_t)SOLVE_FEW * ctx->num_sms;  // eight threads per halo
+  const double rn = rint(ctx->p.n_poly);
+  const bool integer = fabs(ctx->p.n_poly - rn) < 1e-12 && rn >= 1 && rn <= 16;
+  // eight threads per halo
+  const bool few = n <= (int64_t)(integer ? SOLVE_FEW : SOLVE_FEW_POW) * ctx->num_sms;
   const int64_t n8 = NGT * n;
   const int sb8 = bp_item_block(ctx, n8, 128);
   k_setup<<<(unsigned)((n + sb - 1) / sb), sb, 0, ctx->stream>>>(

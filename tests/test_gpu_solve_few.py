@@ -80,3 +80,27 @@ def test_small_catalogues_take_less_time(api):
     print(f"200 halos {few * 1e3:.0f} us, 15000 halos {many * 1e3:.0f} us")
     assert few <= 0.8 * many
     ctx.close()
+
+
+def test_small_catalogues_with_a_fractional_index(api):
+    """Gamma = 1.15 (n = 6.67): 300 halos in less than 0.6 of the solve time of 15000 (0.9 with one
+    thread per halo, 0.4 with eight)."""
+    ctx = api.Context(icm=dict(Gamma=1.15))
+
+    def ms(k):
+        rng = np.random.default_rng(5)
+        a = [cuda(10 ** rng.uniform(12, 15, k)), cuda(rng.uniform(3, 8, k)),
+             cuda(rng.uniform(0.01, 3, k))]
+        ctx.set_timing(True)
+        best = float("inf")
+        for _ in range(20):
+            ctx.phase_times()
+            ctx.solve_halos(*a, raise_on_noconv=False)
+            best = min(best, ctx.phase_times()["solve"])
+        ctx.set_timing(False)
+        return best
+
+    few, many = ms(300), ms(15000)
+    print(f"300 halos {few * 1e3:.0f} us, 15000 halos {many * 1e3:.0f} us")
+    assert few <= 0.6 * many
+    ctx.close()
