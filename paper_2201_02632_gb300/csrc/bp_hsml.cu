@@ -677,7 +677,8 @@ __global__ void __launch_bounds__(32)
       const float R2 = R * R;
       // the particles within R, in tree order
       uint32_t off = 0;
-      search(tree, pc, pc, R2, lane, [&](uint32_t node, unsigned hits, const float4&, const float4&) {
+      search(tree, pc, pc, R2, lane, [&](uint32_t node, unsigned hits, const float4&,
+                                         const float4&) {
         while (hits) {  // four leaves at a time: their loads overlap
           float d2[4];
   #pragma unroll

@@ -52,9 +52,9 @@ __device__ __forceinline__ float gelu_grad(float x) {
 // ([out][in], rows padded to 132 floats: the lanes' 16-byte reads hit all banks whether they
 // run over outputs or inputs).  Warp w owns rows 4 w .. 4 w + 3 of the tile through every layer,
 // so the layers need no CTA barrier; a lane computes 4 rows x 4 outputs (or inputs) and reads 8
-// 16-byte words of shared memory per 64 multiply-adds.  Bound by latency at one tile per SM: 8 warps
-// use 26 to 30% of the issue slots and wait for the weights and the cache (shared-memory reads
-// keep their pipe 25% busy).
+// 16-byte words of shared memory per 64 multiply-adds.  Bound by latency at one tile per SM: 8
+// warps use 26 to 30% of the issue slots and wait for the weights and the cache (shared-memory
+// reads keep their pipe 25% busy).
 // Measured at 4096 rows (one training step of 17 launches took 398 us: the weight gradients ran
 // on 16 CTAs, each layer was a launch, and every activation went through global memory twice):
 // k_forward 20 us (68 us as four launches), k_backward + k_sum_partials 40 us (296 us as

@@ -45,7 +45,8 @@ def test_newton_steps_over_a_clump_and_back(orc, api, ctx, seed, first):
 
 def _cone(n):
     """Light-cone particles, more than one search of the one-warp kernel may meet (65536)."""
-    lc = I.lightcone(n_part=n, n_halo=n // 1333, side_deg=2.0, zr=(0.05, 1.5), seed=I.SEED_BASE + 78)
+    lc = I.lightcone(n_part=n, n_halo=n // 1333, side_deg=2.0, zr=(0.05, 1.5),
+                     seed=I.SEED_BASE + 78)
     return np.stack([lc.parts["x"], lc.parts["y"], lc.parts["z"]])
 
 

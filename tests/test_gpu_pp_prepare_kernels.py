@@ -1,5 +1,5 @@
-"""A pair list prepared for one deposit kernel, deposited by another: bp_pp_deposit asks for the same
-records, geometry and selection, not for the kernel that bp_set_deposit_kernel named before.
+"""A pair list prepared for one deposit kernel, deposited by another: bp_pp_deposit asks for the
+same records, geometry and selection, not for the kernel that bp_set_deposit_kernel named before.
 
 Tolerance: that of every map comparison with the oracle (assert_map_parity)."""
 import numpy as np

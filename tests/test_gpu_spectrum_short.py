@@ -1,5 +1,5 @@
-"""Maps of few rows (several columns per CTA in the second transform) with few and many bins, against
-the oracle with the tolerance of test_gpu_spectrum, and their time."""
+"""Maps of few rows (several columns per CTA in the second transform) with few and many bins,
+against the oracle with the tolerance of test_gpu_spectrum, and their time."""
 import math
 
 import numpy as np
