@@ -681,13 +681,13 @@ __global__ void __launch_bounds__(32)
                                          const float4&) {
         while (hits) {  // four leaves at a time: their loads overlap
           float d2[4];
-  #pragma unroll
+#pragma unroll
           for (int q = 0; q < 4; ++q) {
             d2[q] = INFINITY;
             if (hits) d2[q] = dist2(pos[((uint64_t)node * 32 + __ffs(hits) - 1) * 32 + lane], p);
             hits &= hits - 1;
           }
-  #pragma unroll
+#pragma unroll
           for (int q = 0; q < 4; ++q) {
             const bool in = d2[q] < R2;
             const unsigned m = __ballot_sync(0xffffffffu, in);

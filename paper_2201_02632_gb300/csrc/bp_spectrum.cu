@@ -316,7 +316,7 @@ __global__ void __launch_bounds__(Fft<LG>::T* Fft<LG>::F, Fft<LG>::N <= 4096 ? 2
   // Short columns, several per CTA: a thread per (column, bin), Kahan sums.  (A warp each left two
   // warps 960 turns at 64 columns and 30 bins.  A map of 512 x 2: 482 us before, 47 now; 512 x 128
   // with 256 bins: 310 and 53 us.)
-  if constexpr (F > 1) {
+  if (F > 1 && (N < 256 || nb > 64)) {  // (256 rows, 30 bins: a warp each is 2 us faster)
     each(nb, [&](int ff, int b) {
       if (col0 + ff >= ncol) return;
       const double* p = s_d + (size_t)ff * 2 * P::PADN;
@@ -331,17 +331,20 @@ __global__ void __launch_bounds__(Fft<LG>::T* Fft<LG>::F, Fft<LG>::N <= 4096 ? 2
     });
     return;
   }
-  // a warp per bin
+  // a warp per (column, bin)
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
-  for (int b = wid; b < nb; b += nw) {
-    const int k0 = s_f[0][b], k1 = s_f[0][b + 1];
-    double s = 0.0;
-    for (int k = k0 + lane; k < k1; k += 32) {
-      s += s_d[P::at(k)];
-      if (k > 0 && k < N / 2) s += s_d[P::at(N - k)];
+  for (int ff = 0; ff < F && col0 + ff < ncol; ++ff) {
+    const double* p = s_d + (size_t)ff * 2 * P::PADN;
+    for (int b = wid; b < nb; b += nw) {
+      const int k0 = s_f[ff][b], k1 = s_f[ff][b + 1];
+      double s = 0.0;
+      for (int k = k0 + lane; k < k1; k += 32) {
+        s += p[P::at(k)];
+        if (k > 0 && k < N / 2) s += p[P::at(N - k)];
+      }
+      for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+      if (lane == 0) put(ff, b, s);
     }
-    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-    if (lane == 0) put(0, b, s);
   }
 }
 
@@ -372,7 +375,9 @@ __global__ void __launch_bounds__(BR_THREADS)
   }
   if (t == 0) {
     // norm times the mean in one rounding: the quotient and what it leaves
-    const double n = (double)s_c[0], q = s_s[0] / n, rest = fma(-q, n, s_s[0]) / n;
+    // (1e-16 of it, so that an FP32 reciprocal does for what it leaves)
+    const double n = (double)s_c[0], q = s_s[0] / n;
+    const double rest = fma(-q, n, s_s[0]) * (double)(1.0f / (float)n);
     cl[b] = s_c[0] > 0 ? fma(norm, q, norm * rest) : 0.0;
     if (nmodes) nmodes[b] = s_c[0];
   }
